@@ -199,6 +199,19 @@ struct Plan {
     // pairs of +-|z| (one half of each chunk z <= 0, the other z > 0), so
     // that a chunk's templates have similar widths
     int tc_order = 1;
+    // harmonic sum by bounds (harmonic_bound.cu): the plane's maxima over boxes
+    // of 2 bins x one row block, the blocks' first rows, and per block and
+    // harmonic the source blocks
+    bool pool_on = false;
+    int pool_nb = 0;
+    uint16_t *pool[2] = {nullptr, nullptr};   // [pool_nb][plane_cols / 2] FP16
+    int32_t *pool_blk = nullptr;              // [pool_nb + 1]
+    uint32_t *pool_src = nullptr;             // [pool_nb][H]
+    uint2 *pool_masks = nullptr;              // [pool_nb]
+    // boxes that need their exact sums: (bound, block, box) and their number
+    unsigned long long *pool_list = nullptr;
+    unsigned int pool_list_cap = 0;
+    unsigned int *pool_listed = nullptr;
     // FFT split of the N/2-point complex FFT in the spectrum stage
     int fft_m1, fft_m2;     // M = m1 * m2 (m1 = 1: single pass)
     // device memory
@@ -300,9 +313,17 @@ inline int64_t plane_cols(const Plan &p) { return p.interbin ? 2 * p.n_r : p.n_r
 fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partials,
                                   const double *given_stats, TrialStats *out,
                                   cudaStream_t s);
-fdas_status launch_harmonic_threshold(Plan &p, const void *plane,
+// buf: which of the plan's two planes' workspaces the call may use
+fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf,
                                       const TrialStats *st, uint32_t rank,
                                       cudaStream_t s);
+// the same crossings from bounds on boxes of cells (pool_on plans)
+constexpr int kPoolMaxRows = 4;   // rows of a block
+std::vector<int32_t> pool_blocks(int n_z);
+bool pool_sources(const std::vector<int32_t> &blk, int n_z, int iz0, int H,
+                  std::vector<uint32_t> *src, std::vector<uint32_t> *masks);
+fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, const TrialStats *st,
+                                  uint32_t rank, cudaStream_t s);
 fdas_status launch_harmonic_sums(Plan &p, const void *plane, float *out,
                                  cudaStream_t s);
 fdas_status launch_stuck_wait(unsigned int *flags, long long limit_cycles, cudaStream_t s);

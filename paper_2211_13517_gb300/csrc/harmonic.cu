@@ -15,6 +15,7 @@
 // (trial rank, stage, iz, ir), so the list does not depend on scheduling.
 #include "fdas_internal.cuh"
 #include "fft_cta.cuh"   // cadd
+#include "harmonic_index.cuh"
 #include "tma.cuh"
 #include "check.cuh"
 
@@ -24,8 +25,6 @@
 
 namespace fdas {
 namespace {
-
-constexpr int ilog2h(int n) { return n <= 1 ? 0 : 1 + ilog2h(n >> 1); }
 
 // ---------------------------------------------------------------------------
 // statistics: mean/std from the correlation partials (fixed order) or from a
@@ -40,9 +39,10 @@ struct ThrParams {
 
 __global__ void finalize_stats_kernel(const double2 *__restrict__ partials, int n_partials,
                                       const double *__restrict__ given, TrialStats *out,
-                                      ThrParams tp) {
+                                      ThrParams tp, unsigned int *listed) {
     __shared__ double sa[256], sb[256];
     const int tid = threadIdx.x;
+    if (tid == 0 && listed != nullptr) *listed = 0u;   // boxes of the bound sums that follow
     double a = 0.0, b = 0.0;
     if (given == nullptr) {
         for (int i = tid; i < n_partials; i += 256) {
@@ -99,16 +99,6 @@ __global__ void finalize_stats_kernel(const double2 *__restrict__ partials, int 
 // row exactly (NC * 256 divides N/2), so no load needs a bounds test.
 // ---------------------------------------------------------------------------
 constexpr int kHsThreads = 256;
-
-// harmonic visited at position idx of the stage order
-__host__ __device__ constexpr int j_at(int H, int idx) {
-    return idx == 0 ? H : ((2 * (idx - (1 << ilog2h(idx))) + 1) * H) >> (ilog2h(idx) + 1);
-}
-
-__host__ __device__ constexpr int src_off(int H, int o, int j) {
-    return o < 0 ? -(((-o) * j + H / 2) / H) : ((o * j + H / 2) / H);
-}
-
 
 // element offset of the source row of every harmonic for top row iz (the
 // same for the whole CTA): threads 0..H-1 fill it, then the CTA synchronises
@@ -251,6 +241,10 @@ __global__ void __launch_bounds__(kHsThreads)
 // by 16 bits), adds them to its cells (16-bit planes: one mixed-precision add
 // each), compares each completed stage with its threshold and appends every
 // crossing.
+//
+// kGated: run only when the bound sums (harmonic_bound.cu) listed more boxes
+// than their list holds; the grid is small (it mostly returns at once) and
+// loops over the tiles.
 // ---------------------------------------------------------------------------
 template <class P, int H>
 struct Dedup {
@@ -471,34 +465,40 @@ struct DedupSteps {
     }
 };
 
-template <class P, int H, bool kWriteSums>
+template <class P, int H, bool kWriteSums, bool kGated>
 __global__ void __launch_bounds__(Dedup<P, H>::T, 7)
     harmonic_dedup_kernel(const typename P::real *__restrict__ plane, int64_t n_r, int n_z,
                           int iz0, const TrialStats *__restrict__ st, uint32_t rank,
                           CandRec *__restrict__ cand, unsigned long long *__restrict__ count,
                           int64_t cap, float *__restrict__ sums_out,
-                          unsigned int *__restrict__ flags) {
+                          unsigned int *__restrict__ flags, const unsigned int *__restrict__ gate,
+                          unsigned int gate_cap) {
     using D = Dedup<P, H>;
     using real = typename P::real;
+    // with a gate: only when the bound sums listed more boxes than fit
+    if (kGated && *gate <= gate_cap) return;
     extern __shared__ __align__(16) unsigned char dd_smem[];
     real *sm = reinterpret_cast<real *>(dd_smem);
     using Steps = DedupSteps<P, H>;
     __shared__ __align__(8) uint64_t bars[Steps::NG];
-    const int64_t B = (int64_t)blockIdx.x * D::CELLS;
     const int t = threadIdx.x;
-    const int iz_begin = blockIdx.y * D::QROWS;
-    const int iz_end = min(iz_begin + D::QROWS, n_z);
     if (t == 0) {
         for (int g = 0; g < Steps::NG; ++g) mbar_init(&bars[g], 1);
         mbar_fence_init();
     }
-    const int64_t b = B + (int64_t)D::R * t;   // first cell of this thread
-    const bool active = b < n_r;   // thread 0 always is
     typename Steps::Lane lane_sp;
     if (t < 32) Steps::template lane_span<0>(t, lane_sp);
     const float inv = 1.0f / P::plane_scale;
     bool failed = false;
-    int q = 0;
+    int q = 0;   // rows so far: the barriers' phase
+    const int cols = (int)((n_r + D::CELLS - 1) / D::CELLS);
+    const int n_tiles = cols * ((n_z + D::QROWS - 1) / D::QROWS);
+    for (int tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x) {
+    const int64_t B = (int64_t)(tile % cols) * D::CELLS;
+    const int iz_begin = tile / cols * D::QROWS;
+    const int iz_end = min(iz_begin + D::QROWS, n_z);
+    const int64_t b = B + (int64_t)D::R * t;   // first cell of this thread
+    const bool active = b < n_r;   // thread 0 always is
     uint32_t tv[8];   // 16-bit planes: the thread's top-row cells, one row ahead
     if constexpr (D::kTopRegs)
         if (active && iz_begin < iz_end &&
@@ -517,7 +517,8 @@ __global__ void __launch_bounds__(Dedup<P, H>::T, 7)
             // (their reads by this CTA's threads come before the copies),
             // then one arrival per stage barrier (none on the unused barrier
             // of a top row held in registers)
-            Steps::copy_lane(lane_sp, plane, iz0, iz - iz0, n_r, B, q == 0, sm, bars, n_z);
+            Steps::copy_lane(lane_sp, plane, iz0, iz - iz0, n_r, B, iz == iz_begin, sm,
+                             bars, n_z);
             __syncwarp();
             if (t < Steps::NG && !(t == 0 && D::kTopRegs)) mbar_arrive(&bars[t]);
         }
@@ -574,7 +575,10 @@ __global__ void __launch_bounds__(Dedup<P, H>::T, 7)
         }, tv, next_top);
         if (!ok) failed = true;
     }
-    if (__syncthreads_or(failed)) {
+    failed = __syncthreads_or(failed);
+    if constexpr (!kGated) break;   // one tile per CTA
+    }
+    if (failed) {
         if (t == 0) atomicOr(flags, 2u);
         // copies still in flight must land before the CTA's shared memory
         // is released (each wait bounded): those of the last row issued
@@ -786,25 +790,30 @@ __global__ void finish_kernel(const CandRec *__restrict__ rec, int64_t n_host,
     out[i] = o;
 }
 
-template <class P, int H, bool kWriteSums>
+template <class P, int H, bool kWriteSums, bool kGated>
 fdas_status launch_dedup(Plan &p, const void *plane, const TrialStats *st, uint32_t rank,
                          float *sums_out, cudaStream_t s) {
     using D = Dedup<P, H>;
     const size_t smem = sizeof(typename P::real) * (size_t)D::SMEM_ELEMS;
-    auto k = harmonic_dedup_kernel<P, H, kWriteSums>;
+    auto k = harmonic_dedup_kernel<P, H, kWriteSums, kGated>;
     FDAS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid((unsigned)((p.n_r + D::CELLS - 1) / D::CELLS),
-              (unsigned)((p.n_z + D::QROWS - 1) / D::QROWS));
-    k<<<grid, D::T, smem, s>>>((const typename P::real *)plane, p.n_r, p.n_z, p.iz0, st, rank,
-                               p.cand, p.cand_count, p.store_cap, sums_out, p.flags);
+    int64_t grid = ((p.n_r + D::CELLS - 1) / D::CELLS) * ((p.n_z + D::QROWS - 1) / D::QROWS);
+    if (kGated) grid = std::min<int64_t>(grid, 7 * (int64_t)p.n_sms);   // mostly returns at once
+    k<<<(unsigned)grid, D::T, smem, s>>>((const typename P::real *)plane, p.n_r, p.n_z, p.iz0, st,
+                                         rank, p.cand, p.cand_count, p.store_cap, sums_out, p.flags,
+                                         p.pool_listed, p.pool_list_cap);
     FDAS_CUDA_TRY(cudaGetLastError());
     return FDAS_OK;
 }
 
 template <class P, int H, bool kWriteSums>
 fdas_status launch_hs(Plan &p, const void *plane, const TrialStats *st, uint32_t rank,
-                      float *sums_out, cudaStream_t s) {
-    if constexpr (H <= 16) return launch_dedup<P, H, kWriteSums>(p, plane, st, rank, sums_out, s);
+                      float *sums_out, bool gated, cudaStream_t s) {
+    if constexpr (H <= 16) {
+        if constexpr (!kWriteSums)
+            if (gated) return launch_dedup<P, H, false, true>(p, plane, st, rank, nullptr, s);
+        return launch_dedup<P, H, kWriteSums, false>(p, plane, st, rank, sums_out, s);
+    }
     // cells per thread: as many as the register budget allows (NC * H <= 64)
     // and as divide the row into whole CTAs (N/2 is a power of two >= 512)
     constexpr int NCMAX = H >= 32 ? 2 : 4;
@@ -998,25 +1007,28 @@ fdas_status launch_fund(Plan &p, const void *plane, const TrialStats *st, uint32
 
 template <class P, int H, bool kWriteSums>
 fdas_status launch_hs_mode(Plan &p, const void *plane, const TrialStats *st, uint32_t rank,
-                           float *sums_out, cudaStream_t s) {
+                           float *sums_out, bool gated, cudaStream_t s) {
     if (p.harm_mode == FDAS_HARM_FUNDAMENTAL)
         return launch_fund<P, H, kWriteSums>(p, plane, st, rank, sums_out, s);
-    return launch_hs<P, H, kWriteSums>(p, plane, st, rank, sums_out, s);
+    return launch_hs<P, H, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
 }
 
 template <class P, bool kWriteSums>
 fdas_status launch_hs_P(Plan &p, const void *plane, const TrialStats *st, uint32_t rank,
-                        float *sums_out, cudaStream_t s) {
+                        float *sums_out, bool gated, cudaStream_t s) {
     switch (p.H) {
-        case 1: return launch_hs_mode<P, 1, kWriteSums>(p, plane, st, rank, sums_out, s);
-        case 2: return launch_hs_mode<P, 2, kWriteSums>(p, plane, st, rank, sums_out, s);
-        case 4: return launch_hs_mode<P, 4, kWriteSums>(p, plane, st, rank, sums_out, s);
-        case 8: return launch_hs_mode<P, 8, kWriteSums>(p, plane, st, rank, sums_out, s);
-        case 16: return launch_hs_mode<P, 16, kWriteSums>(p, plane, st, rank, sums_out, s);
-        case 32: return launch_hs_mode<P, 32, kWriteSums>(p, plane, st, rank, sums_out, s);
+        case 1: return launch_hs_mode<P, 1, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
+        case 2: return launch_hs_mode<P, 2, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
+        case 4: return launch_hs_mode<P, 4, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
+        case 8: return launch_hs_mode<P, 8, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
+        case 16: return launch_hs_mode<P, 16, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
+        case 32: return launch_hs_mode<P, 32, kWriteSums>(p, plane, st, rank, sums_out, gated, s);
         default: set_error("bad n_harm"); return FDAS_ERR_ARG;
     }
 }
+
+// shortest row the bound kernels take
+constexpr int64_t kBoundMinCols = 1 << 11;
 
 }  // namespace
 
@@ -1028,25 +1040,27 @@ fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partia
     tp.mode = p.thr_mode;
     tp.n_stages = p.n_stages;
     tp.n_cells = (double)p.n_z * (double)p.n_r;
-    finalize_stats_kernel<<<1, 256, 0, s>>>(partials, n_partials, given_stats, out, tp);
+    finalize_stats_kernel<<<1, 256, 0, s>>>(partials, n_partials, given_stats, out, tp, p.pool_listed);
     FDAS_CUDA_TRY(cudaGetLastError());
     return FDAS_OK;
 }
 
-fdas_status launch_harmonic_threshold(Plan &p, const void *plane, const TrialStats *st,
+fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, const TrialStats *st,
                                       uint32_t rank, cudaStream_t s) {
+    const bool by_bounds = p.pool_on && p.n_r >= kBoundMinCols;
+    if (by_bounds) FDAS_TRY(launch_harmonic_bound(p, plane, buf, st, rank, s));
     switch (p.prec) {
-        case FDAS_FP32: return launch_hs_P<PrecF32, false>(p, plane, st, rank, nullptr, s);
-        case FDAS_BF16: return launch_hs_P<PrecBF16, false>(p, plane, st, rank, nullptr, s);
-        default: return launch_hs_P<PrecF16, false>(p, plane, st, rank, nullptr, s);
+        case FDAS_FP32: return launch_hs_P<PrecF32, false>(p, plane, st, rank, nullptr, by_bounds, s);
+        case FDAS_BF16: return launch_hs_P<PrecBF16, false>(p, plane, st, rank, nullptr, by_bounds, s);
+        default: return launch_hs_P<PrecF16, false>(p, plane, st, rank, nullptr, by_bounds, s);
     }
 }
 
 fdas_status launch_harmonic_sums(Plan &p, const void *plane, float *out, cudaStream_t s) {
     switch (p.prec) {
-        case FDAS_FP32: return launch_hs_P<PrecF32, true>(p, plane, nullptr, 0, out, s);
-        case FDAS_BF16: return launch_hs_P<PrecBF16, true>(p, plane, nullptr, 0, out, s);
-        default: return launch_hs_P<PrecF16, true>(p, plane, nullptr, 0, out, s);
+        case FDAS_FP32: return launch_hs_P<PrecF32, true>(p, plane, nullptr, 0, out, false, s);
+        case FDAS_BF16: return launch_hs_P<PrecBF16, true>(p, plane, nullptr, 0, out, false, s);
+        default: return launch_hs_P<PrecF16, true>(p, plane, nullptr, 0, out, false, s);
     }
 }
 

@@ -148,6 +148,8 @@ constexpr unsigned char kCanary = 0xA5;
 
 cudaError_t bounds_take_harmonic(BoundsLog *out);
 cudaError_t bounds_arm_harmonic(int64_t shrink);
+cudaError_t bounds_take_harmonic_bound(BoundsLog *out);
+cudaError_t bounds_arm_harmonic_bound(int64_t shrink);
 cudaError_t bounds_take_correlate_tc(BoundsLog *out);
 cudaError_t bounds_arm_correlate_tc(int64_t shrink);
 
@@ -206,6 +208,12 @@ static void free_plan_memory(Plan *p) {
         if (p->ev_conv[b]) cudaEventDestroy(p->ev_conv[b]);
         if (p->ev_hsum[b]) cudaEventDestroy(p->ev_hsum[b]);
     }
+    for (int b = 0; b < 2; ++b) dfree(*p, p->pool[b]);
+    dfree(*p, p->pool_blk);
+    dfree(*p, p->pool_src);
+    dfree(*p, p->pool_masks);
+    dfree(*p, p->pool_list);
+    dfree(*p, p->pool_listed);
     dfree(*p, p->stats);
     dfree(*p, p->rank_ids);
     dfree(*p, p->cand);
@@ -289,6 +297,7 @@ static fdas_status debug_check(Plan &p, cudaStream_t s, const std::string &after
         const char *unit;
         cudaError_t (*take)(BoundsLog *);
     } logs[] = {{"harmonic sum", bounds_take_harmonic},
+                {"harmonic sum by bounds", bounds_take_harmonic_bound},
                 {"tensor-core correlation", bounds_take_correlate_tc}};
     for (const auto &l : logs) {
         BoundsLog lg{};
@@ -357,6 +366,7 @@ struct BoundsShrink {
 #ifdef FDAS_CHECK_BOUNDS
         if (want) {
             bounds_arm_harmonic(1);
+            bounds_arm_harmonic_bound(1);
             bounds_arm_correlate_tc(1);
             on = true;
         }
@@ -369,6 +379,7 @@ struct BoundsShrink {
         if (on) {
             cudaDeviceSynchronize();
             bounds_arm_harmonic(0);
+            bounds_arm_harmonic_bound(0);
             bounds_arm_correlate_tc(0);
         }
 #endif
@@ -462,6 +473,21 @@ static Plan plan_view(const Plan &p, int64_t n) {
     v.n_zchunk = choose_zchunks(v, v.n_sms);
     while (v.n_zchunk > 1 && (int64_t)v.n_seg * v.n_zchunk > p.partials_cap) --v.n_zchunk;
     return v;
+}
+
+// Whether the harmonic sum goes by bounds (harmonic_bound.cu).  It adds the
+// pooled plane and two kernels, and pays when few bounds reach a threshold and
+// the plane is more than a few rows: a BF16 search of 2^22 samples x 193 rows,
+// 16 harmonics, against the plain kernel: 6 sigma 738 us (1029), 5.5 sigma 866
+// (1038), 5 sigma 1138 (1072); 8 harmonics: 6 sigma 586 (771), 5 sigma 648
+// (800), 4.5 sigma 1004 (998).  One harmonic only compares cells (308 against
+// 288), and with one row the extra launches cost 10 to 15 us.  Unnormalised
+// planes and the mean + k sigma rule (far lower thresholds) keep the plain
+// kernel.
+static bool bounds_pay(const Plan &p) {
+    return p.harm_mode == FDAS_HARM_TOP && p.H >= 2 && p.H <= 16 && p.n_z >= 12 &&
+           p.norm_mode == FDAS_NORM_MEDIAN && p.thr_mode == FDAS_THRESH_GAMMA_TAIL &&
+           p.sigma >= (p.H == 16 ? 5.4 : 5.0);
 }
 
 static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_max, double z_step,
@@ -654,6 +680,30 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
     // itself and needs only its edge table (allocated below)
     if (p.interbin && p.correlator != FDAS_CORR_TENSOR)
         PLAN_TRY(dalloc(p, &p.corr, cb * (size_t)p.n_z * (size_t)p.n_r, "corr"));
+    {
+        std::vector<uint32_t> src, masks;
+        const std::vector<int32_t> blk = pool_blocks(p.n_z);
+        p.pool_on = bounds_pay(p) && pool_sources(blk, p.n_z, p.iz0, p.H, &src, &masks);
+        if (p.pool_on) {
+            p.pool_nb = (int)blk.size() - 1;
+            const int64_t boxes = (int64_t)p.pool_nb * (plane_cols(p) / 2);
+            p.pool_list_cap = (unsigned)std::max<int64_t>(4096, boxes / 64);
+            for (int b = 0; b < 2; ++b)
+                PLAN_TRY(dalloc(p, &p.pool[b], sizeof(uint16_t) * (size_t)boxes,
+                                b == 0 ? "pool[0]" : "pool[1]"));
+            PLAN_TRY(dalloc(p, &p.pool_list, sizeof(unsigned long long) * p.pool_list_cap, "pool_list"));
+            PLAN_TRY(dalloc(p, &p.pool_listed, sizeof(unsigned int), "pool_listed"));
+            PLAN_TRY(dalloc(p, &p.pool_blk, sizeof(int32_t) * blk.size(), "pool_blk"));
+            PLAN_TRY(dalloc(p, &p.pool_src, sizeof(uint32_t) * src.size(), "pool_src"));
+            PLAN_TRY(dalloc(p, &p.pool_masks, sizeof(uint32_t) * masks.size(), "pool_masks"));
+            PLAN_CUDA(cudaMemcpy(p.pool_masks, masks.data(), sizeof(uint32_t) * masks.size(),
+                                 cudaMemcpyHostToDevice));
+            PLAN_CUDA(cudaMemcpy(p.pool_blk, blk.data(), sizeof(int32_t) * blk.size(),
+                                 cudaMemcpyHostToDevice));
+            PLAN_CUDA(cudaMemcpy(p.pool_src, src.data(), sizeof(uint32_t) * src.size(),
+                                 cudaMemcpyHostToDevice));
+        }
+    }
     PLAN_TRY(grow_stats(p, 64));
     const int64_t rec_cap = next_pow2(p.max_cands);
     PLAN_TRY(dalloc(p, &p.cand, sizeof(CandRec) * (size_t)rec_cap, "cand"));
@@ -996,7 +1046,7 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
         TrialStats *ts = p.stats + rank[t];
         Plan hv = harm_view(v);
         FDAS_TRY(launch_finalize_stats(hv, p.partials[b], plane_partials(v), nullptr, ts, hs));
-        FDAS_TRY(launch_harmonic_threshold(hv, p.plane[b], ts, (uint32_t)rank[t], hs));
+        FDAS_TRY(launch_harmonic_threshold(hv, p.plane[b], b, ts, (uint32_t)rank[t], hs));
         FDAS_DEBUG_CHECK(p, hs, "the harmonic sum of series " + std::to_string(t));
         cudaEvent_t e4 = p.profiling ? mark(hs) : nullptr;
         FDAS_CUDA_TRY(cudaEventRecord(p.ev_hsum[b], hs));
@@ -1517,7 +1567,7 @@ fdas_status fdas_threshold(fdas_plan *plan, const void *plane, const double *sta
     FDAS_CUDA_TRY(cudaMemsetAsync(p.flags, 0, sizeof(unsigned int), s));
     Plan hv = harm_view(p);
     FDAS_TRY(launch_finalize_stats(hv, nullptr, 0, stats, p.stats, s));
-    FDAS_TRY(launch_harmonic_threshold(hv, plane, p.stats, 0, s));
+    FDAS_TRY(launch_harmonic_threshold(hv, plane, 0, p.stats, 0, s));
     const fdas_status st = collect(p, cands, capacity, n_found, s);
     FDAS_DEBUG_CHECK(p, s, "fdas_threshold");
     return st;

@@ -1,0 +1,113 @@
+"""The harmonic sum by bounds (csrc/harmonic_bound.cu) against the plain one.
+
+fdas_threshold on a plan that sums by bounds must return exactly the crossings
+of the sums that fdas_harmonic_sums writes out for the same plane (another
+kernel, which sums every cell): the same cells, bit-identical powers.  The
+statistics given set the thresholds: a mean of 1 on unit-mean planes is the
+search's case (few boxes summed exactly), smaller ones send more boxes to the
+exact sums, and the smallest more than their list holds (the plain kernel takes
+over).
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def capi():
+    import paper_2211_13517_gb300 as pkg
+    pkg.build()
+    from paper_2211_13517_gb300 import capi as c
+    c.lib()
+    return c
+
+
+def _plane(plan, seed, interbin=False):
+    """Exponential cells (unit mean) with bright ones, among them the edges."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    shape = (plan.info.n_z, plan.info.plane_cols)
+    p = -torch.log1p(-torch.rand(shape, generator=g, device="cuda"))
+    r = np.random.RandomState(seed)
+    for _ in range(12):
+        p[r.randint(shape[0]), r.randint(shape[1])] = float(r.uniform(20.0, 300.0))
+    p[0, 0] = p[-1, -1] = p[0, -1] = p[-1, 0] = 60.0
+    p[:, 4:12] = 0.0
+    if plan.info.precision == 2:
+        p = p / 16.0
+    return p.to(plan.spec_dtype)
+
+
+def _check(capi, plan, plane, mean):
+    info = plan.info
+    stats = torch.tensor([mean, mean], dtype=torch.float64, device="cuda")
+    st, c, nf = plan.threshold(plane, stats, capacity=1 << 23)
+    assert st == capi.FDAS_OK and nf == len(c)
+    sums = plan.harmonic_sums(plane)
+    at = 0   # records come ordered by (harm, iz, ir)
+    for s in range(info.n_stages):
+        thr = np.float32(mean * info.stage_factor[s])
+        z, r = torch.nonzero(sums[s] > float(thr), as_tuple=True)
+        mine = c[at:at + len(z)]
+        at += len(z)
+        assert np.all(mine["harm"] == 1 << s)
+        assert np.array_equal(mine["iz"], z.cpu().numpy())
+        assert np.array_equal(mine["ir"], r.cpu().numpy())
+        assert np.array_equal(mine["power"], sums[s][z, r].cpu().numpy())
+    assert at == nf
+    return nf
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("harm", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("n_log2,z_max,z_step", [(12, 0.0, 1.0), (12, 2.0, 1.0), (13, 5.0, 0.5),
+                                                 (15, 96.0, 1.0)])
+def test_threshold_is_the_plain_sums(capi, prec, harm, n_log2, z_max, z_step):
+    plan = capi.Plan(1 << n_log2, 64e-6, z_max, z_step, 2048, harm, precision=prec,
+                     max_candidates=1 << 23)
+    plane = _plane(plan, 10 * n_log2 + harm)
+    found = [_check(capi, plan, plane, mean) for mean in (1.0, 0.6, 0.25)]
+    assert 0 < found[0] <= found[1] <= found[2]
+    # far from unit mean: every box is summed exactly
+    _check(capi, plan, plane * 0.0, 1.0)
+    plan.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_threshold_on_the_half_bin_plane(capi, prec):
+    plan = capi.Plan(1 << 13, 64e-6, 20.0, 1.0, 2048, 8, precision=prec, interbin=True)
+    plane = _plane(plan, 5)
+    assert plane.shape[1] == 1 << 13
+    for mean in (1.0, 0.5):
+        assert _check(capi, plan, plane, mean) > 0
+    plan.close()
+
+
+@pytest.mark.parametrize("corr", [1, 2])
+def test_a_search_with_many_crossings_and_a_short_series(capi, corr):
+    """Bright series of both lengths on one plan: the same records as a plan
+    whose threshold rule keeps the plain kernel, at equal thresholds."""
+    import synthetic as S
+    n = 1 << 15
+    xs = []
+    for m in (n, n // 2, n // 8):
+        x = S.inject_sinusoid(S.white_noise(m, 3), 0.11 * m + 0.2, 3.0, 0.3)
+        xs.append(torch.from_numpy(x).cuda())
+    plan = capi.Plan(n, 64e-6, 24.0, 1.0, 2048, 16, precision=1, correlator=corr)
+    st, c, nf = plan.search(xs, capacity=1 << 18)
+    assert st == capi.FDAS_OK and nf == len(c) > 100
+    # each series alone, through the stages
+    for t, x in enumerate(xs):
+        sub = capi.Plan(x.numel(), 64e-6, 24.0, 1.0, 2048, 16, precision=1, correlator=corr)
+        plane, stats = sub.power_plane(sub.spectrum(x))
+        st1, c1, n1 = sub.threshold(plane, stats, capacity=1 << 18)
+        mine = c[c["trial_id"] == t]
+        assert st1 == capi.FDAS_OK and n1 == len(mine)
+        for k in ("harm", "iz", "ir", "power"):
+            assert np.array_equal(mine[k], c1[k]), k
+        mean = float(stats[0])
+        assert _check(capi, sub, plane, mean) == n1
+        sub.close()
+    plan.close()
