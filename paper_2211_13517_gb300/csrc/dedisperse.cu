@@ -43,6 +43,7 @@ constexpr int kDdThreads = 256;  // 8 warps x 4 DM trials
 constexpr int kDdPer = kDdT / 32;
 constexpr double kDm = 4.148808e3;
 constexpr size_t kDdSmemCap = 200 * 1024;   // both buffers
+constexpr size_t kGrSmem = 220 * 1024;      // by groups: all CTAs of an SM
 
 __global__ void dm_delay_kernel(int32_t *__restrict__ out, int n_chan, int n_dm, double f_top,
                                 double df, double tsamp, double dm_lo, double dm_step) {
@@ -200,6 +201,361 @@ __global__ void __launch_bounds__(kDdThreads, 2)
     }
 }
 
+// ---------------------------------------------------------------------------
+// Dedispersion by channel groups.
+//
+// The delays of up to 4 neighbouring channels differ by a few samples, and
+// over the 32 DM trials of a tile they do so in only a few ways: a "pattern"
+// is the tuple of the channels' shifts relative to the first one (3.7 patterns
+// per group of 4 on average for 1024 channels of 0.25 MHz below 1670 MHz and 32
+// trials 0.25 pc cm^-3 apart).  So the channels of a group are summed once per
+// pattern into shared memory, and every DM trial adds one value per group
+// instead of one per channel: the plain kernel's bound, one shared-memory load
+// per addition, falls by nearly the group's size.
+//
+// A CTA owns 32 DM trials x 512 output samples, as the plain kernel does.  Per
+// batch of groups: the windows of the batch's channels arrive by asynchronous
+// copies (the next batch's are in flight meanwhile); the warps form the
+// pattern sums, sorted so that a pattern keeps the partial sums of the leading
+// channels it shares with the one before; then warp w adds to the DM trials
+// 4w .. 4w+3 at each trial's offset.  FP32: sums of a group's channels in
+// channel order, groups in order.  8-bit: sums as pairs of 16-bit integers (two
+// samples per word and addition), stored twice, the second time one sample
+// further on, so that odd offsets find aligned words too; 32-bit totals every
+// 64 groups (64 * 4 * 255 < 2^16).  Exact.
+//
+// Bound: instruction issue (about 2.1 per cycle), half of it the pattern sums.
+// Measured: 1024 channels of 8-bit samples, 128 trials, 2^20 outputs 7.35 ms
+// (plain kernel 18.7); 300 FP32 channels, 75 trials, 262181 outputs 0.63 ms
+// (1.32).
+// ---------------------------------------------------------------------------
+constexpr int kGrMax = 4;         // channels per group
+constexpr int kGrPat = 8;         // patterns per group
+constexpr int kGrBatchMax = 8;    // groups per batch
+constexpr int kGrFlush = 64;      // groups between 32-bit totals (8-bit samples)
+// samples of a pattern sum that a warp forms at a time
+template <class T>
+constexpr int kGrCtas = sizeof(T) == 4 ? 2 : 3;   // CTAs per SM
+template <class T>
+constexpr int kGrChunk = sizeof(T) == 4 ? 160 : 248;
+constexpr int kGrPer = 5;         // FP32 samples of a chunk per lane
+
+// one group of a DM tile as the kernel reads it (whole 16-byte copies)
+struct GrRec {
+    int32_t c0, nk, np, pad;      // first channel, channels, patterns
+    int16_t pat[kGrPat][4];       // [0]: first channel that differs from the pattern
+                                  // before; [k]: shift of channel k
+    // per DM the first word of its samples among the group's pattern sums, of
+    // FP32 and of 8-bit samples (words of two; odd offsets in the second copy)
+    int32_t off[2][kDdD];
+};
+static_assert(sizeof(GrRec) % 16 == 0, "whole 16-byte copies");
+
+// 8 samples (four 16-bit pairs) of an 8-bit window from byte `at` + 8 lane on
+__device__ __forceinline__ void add8_u8(const uint8_t *x, int at, int lane, uint32_t (&v)[4]) {
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(x) + (at >> 2) + 2 * lane;
+    const uint32_t a = w[0], b = w[1], c = w[2];
+    const unsigned sh = 8u * (unsigned)(at & 3);
+    const uint32_t lo = __funnelshift_r(a, b, sh), hi = __funnelshift_r(b, c, sh);
+    v[0] += __byte_perm(lo, 0u, 0x4140u);
+    v[1] += __byte_perm(lo, 0u, 0x4342u);
+    v[2] += __byte_perm(hi, 0u, 0x4140u);
+    v[3] += __byte_perm(hi, 0u, 0x4342u);
+}
+
+// shared-memory geometry: per slot the channel windows (xpitch bytes each) and
+// the batch's records; then the pattern sums (ypitch words each)
+template <class T>
+__global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
+    dedisperse_group_kernel(const T *__restrict__ fb, const int32_t *__restrict__ delays,
+                            const GrRec *__restrict__ recs, const int32_t *__restrict__ n_groups,
+                            int max_groups, float *__restrict__ out, int n_chan, int64_t n_t,
+                            int n_dm, int64_t n_out, int chunks, int lead, int xpitch, int ypitch,
+                            int max_pat, int batch) {
+    constexpr bool kU8 = sizeof(T) == 1;
+    extern __shared__ __align__(16) unsigned char dd_smem[];
+    const int slot_bytes = batch * (kGrMax * xpitch + (int)sizeof(GrRec));
+    uint32_t *const Y = reinterpret_cast<uint32_t *>(dd_smem + 2 * slot_bytes);
+    __shared__ int32_t shift[2][kGrBatchMax * kGrMax];   // of each window's first sample
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t0 = (int64_t)blockIdx.x * kDdT;
+    const int d_lo = blockIdx.y * kDdD;
+    const int32_t *dl = delays + (int64_t)d_lo * n_chan;
+    const GrRec *rec = recs + (int64_t)blockIdx.y * max_groups;
+    const int ng = n_groups[blockIdx.y];
+    auto slot_rec = [&](int slot) {
+        return reinterpret_cast<const GrRec *>(dd_smem + slot * slot_bytes +
+                                               batch * kGrMax * xpitch);
+    };
+    auto stage = [&](int g0, int slot) {
+        const int n = min(batch, ng - g0);
+        unsigned char *base = dd_smem + slot * slot_bytes;
+        unsigned char *rd = base + batch * kGrMax * xpitch;
+        for (int i = threadIdx.x; i < n * (int)(sizeof(GrRec) / 16); i += kDdThreads)
+            cp_async16(rd + 16 * i, reinterpret_cast<const unsigned char *>(rec + g0) + 16 * i, 16);
+        // one warp per channel
+        for (int i = warp; i < n * kGrMax; i += kDdThreads / 32) {
+            const int g = i / kGrMax, k = i % kGrMax;
+            if (k >= __ldg(&rec[g0 + g].nk)) continue;
+            const int c = __ldg(&rec[g0 + g].c0) + k;
+            // the window starts `lead` samples early (shifts may be negative),
+            // rounded down to an address of a multiple of 16 bytes
+            const int64_t first = t0 + __ldg(dl + c) - lead;
+            const T *src = fb + (int64_t)c * n_t;
+            constexpr int kV = 16 / (int)sizeof(T);
+            const int a = (int)((reinterpret_cast<uintptr_t>(src + first) / sizeof(T)) % kV);
+            T *dst = reinterpret_cast<T *>(base + i * xpitch);
+            if (lane == 0) shift[slot][i] = lead + a;
+            if (first - a >= 0 && first - a + xpitch / (int)sizeof(T) <= n_t) {
+                const T *from = src + (first - a);
+                for (int j = lane; j < xpitch / 16; j += 32)
+                    cp_async16(dst + kV * j, from + kV * j, 16);
+                continue;
+            }
+            for (int j = lane; j < xpitch / 16; j += 32) {
+                const int64_t s = first - a + kV * j;
+                if (s >= 0) {
+                    const int64_t left = n_t - s;
+                    const int valid = left <= 0 ? 0 : (left >= kV ? 16 : (int)left * (int)sizeof(T));
+                    cp_async16(dst + kV * j, src + (valid > 0 ? s : 0), valid);
+                } else {
+                    // before the first sample: zeros, then element by element
+#pragma unroll
+                    for (int x = 0; x < kV; ++x)
+                        dst[kV * j + x] = s + x >= 0 && s + x < n_t ? src[s + x] : (T)0;
+                }
+            }
+        }
+        cp_async_commit();
+    };
+
+    // 8-bit: the 32-bit totals, touched every 64 groups only, stay in local
+    // memory (reached through a pointer the compiler cannot see through), which
+    // leaves the registers for a third CTA per SM
+    using Acc = typename DdIn<T>::Acc;
+    Acc acc[4][kDdPer];
+    Acc *total = &acc[0][0];
+    if constexpr (kU8) asm volatile("" : "+l"(total) : : "memory");
+    uint32_t part[4][kU8 ? kDdPer / 2 : 1];   // 8-bit: pairs of 16-bit partial sums
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int k = 0; k < kDdPer; ++k) {
+            if constexpr (kU8) total[q * kDdPer + k] = 0;
+            else acc[q][k] = 0;
+        }
+#pragma unroll
+        for (int k = 0; k < (kU8 ? kDdPer / 2 : 1); ++k) part[q][k] = 0u;
+    }
+    const bool warp_on = d_lo + 4 * warp < n_dm;
+    int since = 0;   // groups in `part`
+    auto flush = [&] {
+        if constexpr (kU8) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int k = 0; k < kDdPer / 2; ++k) {
+                    total[q * kDdPer + 2 * k] += (int)(part[q][k] & 0xffffu);
+                    total[q * kDdPer + 2 * k + 1] += (int)(part[q][k] >> 16);
+                    part[q][k] = 0u;
+                }
+            since = 0;
+        }
+    };
+
+    stage(0, 0);
+    int slot = 0;
+    for (int g0 = 0; g0 < ng; g0 += batch, slot ^= 1) {
+        const int n = min(batch, ng - g0);
+        cp_async_wait<0>();
+        __syncthreads();   // this batch has landed; every warp is done with the sums before
+        if (g0 + batch < ng) stage(g0 + batch, slot ^ 1);
+        const GrRec *r = slot_rec(slot);
+        // pattern sums: one warp per group and kGrChunk samples
+        for (int it = warp; it < n * chunks; it += kDdThreads / 32) {
+            const int g = it / chunks, ch = it - g * chunks;
+            const int np = r[g].np, nk = r[g].nk;
+            const unsigned char *xs = dd_smem + slot * slot_bytes + g * kGrMax * xpitch;
+            const int32_t *sh = shift[slot] + g * kGrMax;
+            if constexpr (!kU8) {
+                // lane: samples chunk start + lane + 32 j
+                const float *xw = reinterpret_cast<const float *>(xs) + kGrChunk<T> * ch + lane;
+                float *y = reinterpret_cast<float *>(Y) + g * max_pat * ypitch + kGrChunk<T> * ch + lane;
+                float p0[kGrPer], p1[kGrPer], p2[kGrPer];
+                {
+                    const float *w = xw + sh[0];
+#pragma unroll
+                    for (int j = 0; j < kGrPer; ++j) p0[j] = w[32 * j];
+                }
+                // v = u + channel k at shift s (u itself past the group's channels)
+                auto x = [&](int k, int s, const float (&u)[kGrPer], float (&v)[kGrPer]) {
+                    if (k < nk) {
+                        const float *w = xw + k * (xpitch / 4) + sh[k] + s;
+#pragma unroll
+                        for (int j = 0; j < kGrPer; ++j) v[j] = u[j] + w[32 * j];
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < kGrPer; ++j) v[j] = u[j];
+                    }
+                };
+                for (int p = 0; p < np; ++p, y += ypitch) {
+                    const short4 pt = *reinterpret_cast<const short4 *>(r[g].pat[p]);
+                    if (pt.x <= 1) x(1, pt.y, p0, p1);
+                    if (pt.x <= 2) x(2, pt.z, p1, p2);
+                    float v[kGrPer];
+                    x(3, pt.w, p2, v);
+#pragma unroll
+                    for (int j = 0; j < kGrPer; ++j) y[32 * j] = v[j];
+                }
+            } else {
+                // lane: samples 248 ch + 8 lane .. + 7 as four pairs; lane 31 only
+                // hands its first sample to lane 30
+                uint32_t *y = Y + g * max_pat * 2 * ypitch + 124 * ch + 4 * lane;
+                uint32_t p0[4] = {0u, 0u, 0u, 0u}, p1[4], p2[4];
+                add8_u8(xs, sh[0] + 248 * ch, lane, p0);
+                auto x = [&](int k, int s, const uint32_t (&u)[4], uint32_t (&v)[4]) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[j] = u[j];
+                    if (k < nk) add8_u8(xs + k * xpitch, sh[k] + s + 248 * ch, lane, v);
+                };
+                for (int p = 0; p < np; ++p, y += 2 * ypitch) {
+                    const short4 pt = *reinterpret_cast<const short4 *>(r[g].pat[p]);
+                    if (pt.x <= 1) x(1, pt.y, p0, p1);
+                    if (pt.x <= 2) x(2, pt.z, p1, p2);
+                    uint32_t v[4];
+                    x(3, pt.w, p2, v);
+                    const uint32_t nx = __shfl_down_sync(0xffffffffu, v[0], 1);
+                    if (lane < 31) {
+                        *reinterpret_cast<uint4 *>(y) = make_uint4(v[0], v[1], v[2], v[3]);
+                        // and one sample further on
+                        *reinterpret_cast<uint4 *>(y + ypitch) = make_uint4(
+                            __byte_perm(v[0], v[1], 0x5432u), __byte_perm(v[1], v[2], 0x5432u),
+                            __byte_perm(v[2], v[3], 0x5432u), __byte_perm(v[3], nx, 0x5432u));
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (!warp_on) continue;
+        if constexpr (!kU8) {
+            for (int g = 0; g < n; ++g) {
+                const int4 o = *reinterpret_cast<const int4 *>(r[g].off[0] + 4 * warp);
+                const float *y = reinterpret_cast<const float *>(Y) + g * max_pat * ypitch + lane;
+                add_pair(y, o.x, o.y, acc[0], acc[1]);
+                add_pair(y, o.z, o.w, acc[2], acc[3]);
+            }
+        } else {
+            // two groups per addition
+            const uint32_t *y = Y + lane;
+            const int per = 2 * max_pat * ypitch;
+            int g = 0;
+            for (; g + 1 < n; g += 2) {
+                const int4 oa = *reinterpret_cast<const int4 *>(r[g].off[1] + 4 * warp);
+                const int4 ob = *reinterpret_cast<const int4 *>(r[g + 1].off[1] + 4 * warp);
+                const int wa[4] = {oa.x, oa.y, oa.z, oa.w}, wb[4] = {ob.x, ob.y, ob.z, ob.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t *a = y + g * per + wa[q], *b = y + (g + 1) * per + wb[q];
+#pragma unroll
+                    for (int k = 0; k < kDdPer / 2; ++k) part[q][k] += a[32 * k] + b[32 * k];
+                }
+            }
+            if (g < n) {
+                const int4 oa = *reinterpret_cast<const int4 *>(r[g].off[1] + 4 * warp);
+                const int wa[4] = {oa.x, oa.y, oa.z, oa.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t *a = y + g * per + wa[q];
+#pragma unroll
+                    for (int k = 0; k < kDdPer / 2; ++k) part[q][k] += a[32 * k];
+                }
+            }
+            since += n;
+            if (since > kGrFlush - kGrBatchMax) flush();
+        }
+    }
+    flush();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int d = d_lo + 4 * warp + q;
+        if (d >= n_dm) continue;
+        float *row = out + (int64_t)d * n_out;
+#pragma unroll
+        for (int k = 0; k < kDdPer; ++k) {
+            const int64_t t = kU8 ? t0 + 2 * (lane + 32 * (k >> 1)) + (k & 1) : t0 + lane + 32 * k;
+            if (t < n_out) row[t] = (float)(kU8 ? total[q * kDdPer + k] : acc[q][k]);
+        }
+    }
+}
+
+// The groups of one DM tile (rows d0 .. d1 - 1 of the delay table): runs of up
+// to 4 channels, halved until their trials' shifts form at most kGrPat
+// patterns.
+struct GrShape {
+    int lo = 0, hi = 0;   // smallest and largest shift
+    double cost = 0.0;    // shared-memory accesses per 32 samples
+};
+void group_tile(const int32_t *delays, int n_chan, int d0, int d1, int chunks, std::vector<GrRec> &out,
+                GrShape &shape) {
+    for (int c = 0; c < n_chan;) {
+        int nk = std::min(kGrMax, n_chan - c);
+        for (;; nk = nk / 2) {
+            struct Pat {
+                int s[kGrMax];
+            };
+            std::vector<Pat> pats;
+            const int nd = d1 - d0;
+            std::vector<Pat> of(nd);
+            const int32_t *base = delays + (size_t)d0 * n_chan + c;
+            for (int d = 0; d < nd; ++d) {
+                const int32_t *row = delays + (size_t)(d0 + d) * n_chan + c;
+                for (int k = 0; k < kGrMax; ++k)
+                    of[d].s[k] = k < nk ? (row[k] - base[k]) - (row[0] - base[0]) : 0;
+            }
+            pats = of;
+            auto less = [](const Pat &a, const Pat &b) {
+                return std::lexicographical_compare(a.s, a.s + kGrMax, b.s, b.s + kGrMax);
+            };
+            auto same = [](const Pat &a, const Pat &b) { return std::equal(a.s, a.s + kGrMax, b.s); };
+            std::sort(pats.begin(), pats.end(), less);
+            pats.erase(std::unique(pats.begin(), pats.end(), same), pats.end());
+            bool fits = (int)pats.size() <= kGrPat;
+            for (const Pat &q : pats)
+                for (int k = 1; k < nk; ++k) fits = fits && q.s[k] >= -64 && q.s[k] <= 64;
+            if (!fits && nk > 1) continue;
+            GrRec r{};
+            r.c0 = c;
+            r.nk = nk;
+            r.np = (int)pats.size();
+            int nodes = 1;
+            for (int p = 0; p < r.np; ++p) {
+                int first = 1;
+                if (p > 0)
+                    while (first < kGrMax && pats[p].s[first] == pats[p - 1].s[first]) ++first;
+                r.pat[p][0] = (int16_t)first;
+                for (int k = 1; k < kGrMax; ++k) r.pat[p][k] = (int16_t)pats[p].s[k];
+                nodes += std::max(0, nk - first);
+                for (int k = 1; k < nk; ++k) {
+                    shape.lo = std::min(shape.lo, pats[p].s[k]);
+                    shape.hi = std::max(shape.hi, pats[p].s[k]);
+                }
+            }
+            for (int d = 0; d < kDdD; ++d) {
+                const int dd = std::min(d, nd - 1);
+                const int p = (int)(std::lower_bound(pats.begin(), pats.end(), of[dd], less) -
+                                    pats.begin());
+                const int off = delays[(size_t)(d0 + dd) * n_chan + c] - base[0];
+                r.off[0][d] = p;     // (turned into words once the layout is known)
+                r.off[1][d] = off;
+            }
+            shape.cost += 4.0 * chunks * (nodes + r.np) + 16.0 * nd;
+            out.push_back(r);
+            break;
+        }
+        c += out.back().nk;
+    }
+}
+
 }  // namespace
 
 struct DedispPlan {
@@ -210,20 +566,70 @@ struct DedispPlan {
     std::vector<int32_t> host_delays;
     int32_t max_delay = 0, span = 0, win = 0, chan_batch = 0, chan_batch_u8 = 0;
     int device = 0;
+    // channel groups: used when they need fewer shared-memory accesses than
+    // the plain kernel's one per addition (few channels with widely different
+    // delays leave groups of one channel)
+    bool grouped = false;
+    GrRec *recs = nullptr;          // device [tiles][max_groups]
+    int32_t *n_groups = nullptr;    // device [tiles]
+    int32_t max_groups = 0, max_pat = 1, lead = 0, tail = 0;
+    int64_t table_bytes = 0;
 };
+
+// bytes of a channel window, words of a pattern sum and groups per batch
+template <class T>
+static void group_layout(const DedispPlan &p, int *chunks, int *xpitch, int *ypitch, int *batch,
+                         size_t *smem) {
+    *chunks = (kDdT + p.span + kGrChunk<T> - 1) / kGrChunk<T>;
+    // samples a window is read over, from up to 15 bytes past a 16-byte boundary
+    // (8-bit: lane 31's samples and a word past them too)
+    const int len = kGrChunk<T> * *chunks + p.lead + p.tail + (sizeof(T) == 4 ? 3 : 15 + 16);
+    *xpitch = ((int)sizeof(T) * len + 15) / 16 * 16;
+    *ypitch = sizeof(T) == 4 ? kGrChunk<T> * *chunks : (kGrChunk<T> / 2) * *chunks;
+    const size_t per = 2 * (kGrMax * (size_t)*xpitch + sizeof(GrRec)) +
+                       4 * (size_t)p.max_pat * *ypitch * (sizeof(T) == 4 ? 1 : 2);
+    // as many groups as fill the warps of the pattern sums best
+    const int warps = kDdThreads / 32, most = (int)std::min<size_t>(kGrBatchMax, kGrSmem / kGrCtas<T> / per);
+    *batch = 0;
+    double best = 0.0;
+    for (int b = 1; b <= most; ++b) {
+        const double fill = (double)b * *chunks / (warps * ((b * *chunks + warps - 1) / warps));
+        if (fill >= best) {
+            best = fill;
+            *batch = b;
+        }
+    }
+    *smem = per * (size_t)*batch;
+}
 
 template <class T>
 fdas_status launch_dedisperse(DedispPlan &p, const T *filterbank, float *out, cudaStream_t s) {
     int cur = 0;
     cudaGetDevice(&cur);
     if (cur != p.device) cudaSetDevice(p.device);
+    dim3 grid((unsigned)((p.n_out + kDdT - 1) / kDdT), (unsigned)((p.n_dm + kDdD - 1) / kDdD));
+    cudaError_t e;
+    if (p.grouped) {
+        int chunks, xpitch, ypitch, batch;
+        size_t smem;
+        group_layout<T>(p, &chunks, &xpitch, &ypitch, &batch, &smem);
+        e = cudaFuncSetAttribute(dedisperse_group_kernel<T>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) {
+            dedisperse_group_kernel<T><<<grid, kDdThreads, smem, s>>>(
+                filterbank, p.delays, p.recs, p.n_groups, p.max_groups, out, p.n_chan, p.n_t, p.n_dm,
+                p.n_out, chunks, p.lead, xpitch, ypitch, p.max_pat, batch);
+            e = cudaGetLastError();
+        }
+        if (cur != p.device) cudaSetDevice(cur);
+        return e == cudaSuccess ? FDAS_OK : cuda_status(e, "dedisperse_group_kernel");
+    }
     const int pitch = p.win + DdIn<T>::kPad;
     const int cb = sizeof(T) == 4 ? p.chan_batch : p.chan_batch_u8;
     const size_t smem = 2 * sizeof(T) * (size_t)pitch * cb;
-    cudaError_t e = cudaFuncSetAttribute(dedisperse_kernel<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(dedisperse_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
     if (e == cudaSuccess) {
-        dim3 grid((unsigned)((p.n_out + kDdT - 1) / kDdT), (unsigned)((p.n_dm + kDdD - 1) / kDdD));
         dedisperse_kernel<T><<<grid, kDdThreads, smem, s>>>(filterbank, p.delays, out, p.n_chan,
                                                             p.n_t, p.n_dm, p.n_out, p.win, cb);
         e = cudaGetLastError();
@@ -282,6 +688,8 @@ fdas_status fdas_dedisp_plan_create(fdas_dedisp_plan **out, int32_t n_chan, int6
         p->dm_step = dm_step;
         auto fail = [&](fdas_status s) {
             cudaFree(p->delays);
+            cudaFree(p->recs);
+            cudaFree(p->n_groups);
             delete p;
             return s;
         };
@@ -325,6 +733,60 @@ fdas_status fdas_dedisp_plan_create(fdas_dedisp_plan **out, int32_t n_chan, int6
         // 8-bit windows: a quarter of the bytes, so more channels per batch
         const size_t per_chan_u8 = 2 * (size_t)(p->win + 16);
         p->chan_batch_u8 = (int)std::max<size_t>(1, std::min<size_t>(16, (96 * 1024) / per_chan_u8));
+        // channel groups per DM tile
+        {
+            const int tiles = (n_dm + fdas::kDdD - 1) / fdas::kDdD;
+            const int chunks = (fdas::kDdT + span + 127) / 128;
+            std::vector<std::vector<fdas::GrRec>> per(tiles);
+            std::vector<int32_t> counts(tiles);
+            fdas::GrShape shape;
+            double plain = 0.0;
+            size_t most = 0;
+            for (int t = 0; t < tiles; ++t) {
+                const int d0 = t * fdas::kDdD, d1 = std::min(n_dm, d0 + fdas::kDdD);
+                fdas::group_tile(p->host_delays.data(), n_chan, d0, d1, chunks, per[t], shape);
+                plain += 16.0 * (d1 - d0) * n_chan;
+                counts[t] = (int32_t)per[t].size();
+                most = std::max(most, per[t].size());
+                for (const fdas::GrRec &r : per[t]) p->max_pat = std::max(p->max_pat, r.np);
+            }
+            p->lead = -shape.lo;
+            p->tail = shape.hi;
+            int nc, xp, ypf, ypu, bf, bu;
+            size_t sm;
+            fdas::group_layout<float>(*p, &nc, &xp, &ypf, &bf, &sm);
+            fdas::group_layout<uint8_t>(*p, &nc, &xp, &ypu, &bu, &sm);
+            // (accesses of the pattern sums and of the trials against the plain
+            // kernel's one per addition; at equal counts the extra barriers and
+            // table reads make groups slower)
+            if (shape.cost < 0.75 * plain && bf >= 1 && bu >= 1 && span < (1 << 24)) {
+                std::vector<fdas::GrRec> flat(most * (size_t)tiles);
+                for (int t = 0; t < tiles; ++t)
+                    std::copy(per[t].begin(), per[t].end(), flat.begin() + (size_t)t * most);
+                for (fdas::GrRec &r : flat)
+                    for (int d = 0; d < fdas::kDdD; ++d) {
+                        const int pat = r.off[0][d], off = r.off[1][d];
+                        r.off[0][d] = pat * ypf + off;
+                        r.off[1][d] = (2 * pat + (off & 1)) * ypu + off / 2;
+                    }
+                p->table_bytes = (int64_t)(sizeof(fdas::GrRec) * flat.size() + sizeof(int32_t) * tiles);
+                e = cudaMalloc(&p->recs, sizeof(fdas::GrRec) * flat.size());
+                if (e == cudaSuccess) e = cudaMalloc(&p->n_groups, sizeof(int32_t) * tiles);
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    fdas::set_error("dedispersion: out of device memory for the channel groups");
+                    return fail(FDAS_ERR_OOM);
+                }
+                e = cudaMemcpy(p->recs, flat.data(), sizeof(fdas::GrRec) * flat.size(),
+                               cudaMemcpyHostToDevice);
+                if (e == cudaSuccess)
+                    e = cudaMemcpy(p->n_groups, counts.data(), sizeof(int32_t) * tiles,
+                                   cudaMemcpyHostToDevice);
+                if (e != cudaSuccess) return fail(fdas::cuda_status(e, "cudaMemcpy"));
+                p->max_groups = (int32_t)most;
+                p->grouped = true;
+            }
+        }
         *out = reinterpret_cast<fdas_dedisp_plan *>(p);
         return FDAS_OK;
     } catch (...) {
@@ -337,6 +799,8 @@ void fdas_dedisp_plan_destroy(fdas_dedisp_plan *plan) {
     if (!plan) return;
     DedispPlan *p = reinterpret_cast<DedispPlan *>(plan);
     cudaFree(p->delays);
+    cudaFree(p->recs);
+    cudaFree(p->n_groups);
     delete p;
 }
 
@@ -354,7 +818,7 @@ fdas_status fdas_dedisp_get_info(const fdas_dedisp_plan *plan, fdas_dedisp_info 
     info->dm_step = p.dm_step;
     info->max_delay = p.max_delay;
     info->tile_span = p.span;
-    info->workspace_bytes = (int64_t)sizeof(int32_t) * p.n_chan * p.n_dm;
+    info->workspace_bytes = (int64_t)sizeof(int32_t) * p.n_chan * p.n_dm + p.table_bytes;
     return FDAS_OK;
 }
 
