@@ -352,9 +352,9 @@ fdas_status launch_prec(Plan &p, const void *spec_padded, void *plane, double2 *
 }
 
 fdas_status launch_correlate(Plan &p, const void *spec_padded, void *plane, double2 *partials,
-                             cudaStream_t s, bool cplx) {
+                             cudaStream_t s, bool cplx, uint16_t *pool) {
     if (p.correlator == FDAS_CORR_TENSOR)
-        return launch_correlate_tc(p, spec_padded, plane, partials, s, cplx);
+        return launch_correlate_tc(p, spec_padded, plane, partials, s, cplx, pool);
     return cplx ? launch_prec<true>(p, spec_padded, plane, partials, s)
                 : launch_prec<false>(p, spec_padded, plane, partials, s);
 }

@@ -66,6 +66,9 @@ constexpr int kTcStages = 4;                     // spectrum-window ring
 constexpr int kTcEpiWarps = 8;
 constexpr int kTcZpt = kTcZ / (kTcEpiWarps / 4);   // templates per epilogue thread
 static_assert(kTcZ % (kTcEpiWarps / 4) == 0, "epilogue split");
+// row blocks of a full part of 14 templates: 3, 4, 3 and 4 rows
+constexpr unsigned kTcFullEnds = (1u << 2) | (1u << 6) | (1u << 9) | (1u << 13);
+static_assert(kTcZpt == 14, "row blocks of a part");
 constexpr int kTcThreads = 32 * (2 + kTcEpiWarps);
 constexpr int kTcTmemCols = 512;
 constexpr int kTcAccStride = 256;                // TMEM column of accumulator 1
@@ -104,6 +107,68 @@ __device__ __forceinline__ float2 fsub2(float2 a, float2 b) {
 }
 
 enum { kPower = 0, kCplx = 1, kInterbin = 2 };
+
+// Two boxes as an FP16 pair, from the row block's maxima: of 16-bit planes the
+// stored cells (a box's two cells in one word), of FP32 ones the boxes' maxima.
+template <class P>
+__device__ __forceinline__ uint32_t pool_pair(uint32_t a, uint32_t b) {
+    __half2 h;
+    if constexpr (P::id == FDAS_FP32) {
+        h = __floats2half2_rn(__uint_as_float(a), __uint_as_float(b));
+    } else {
+        const uint32_t e = __vmaxs2(__byte_perm(a, b, 0x5410u), __byte_perm(a, b, 0x7632u));
+        if constexpr (P::id == FDAS_BF16) {
+            h = __floats2half2_rn(__uint_as_float(e << 16), __uint_as_float(e & 0xffff0000u));
+        } else {
+            memcpy(&h, &e, 4);
+            h = __hmul2(h, __float2half2_rn(1.0f / P::plane_scale));
+        }
+    }
+    uint32_t w;
+    memcpy(&w, &h, 4);
+    return w;
+}
+
+// Maxima of the first W words of v over the row blocks of a part's templates
+// (bit k of `ends`: template k is the last of a block), each handed to
+// put(block, maxima).  Cells are >= 0, so their bit patterns order as signed
+// integers (W words of one FP32 value each with kF32, else of two 16-bit ones).
+template <int W, bool kF32 = false, class F>
+__device__ __forceinline__ void pool_blocks_of(const uint32_t (&v)[kTcZpt][8], unsigned ends,
+                                               const F &put) {
+    auto max3 = [](uint32_t a, uint32_t b, uint32_t c) {
+        if constexpr (kF32) return (uint32_t)__vimax3_s32((int)a, (int)b, (int)c);
+        return __vimax3_s16x2(a, b, c);
+    };
+    if (ends == kTcFullEnds) {   // a full part: blocks of 3, 4, 3 and 4
+        uint32_t m[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) m[w] = max3(v[0][w], v[1][w], v[2][w]);
+        put(0, m);
+#pragma unroll
+        for (int w = 0; w < W; ++w) m[w] = max3(max3(v[3][w], v[4][w], v[5][w]), v[6][w], v[6][w]);
+        put(1, m);
+#pragma unroll
+        for (int w = 0; w < W; ++w) m[w] = max3(v[7][w], v[8][w], v[9][w]);
+        put(2, m);
+#pragma unroll
+        for (int w = 0; w < W; ++w) m[w] = max3(max3(v[10][w], v[11][w], v[12][w]), v[13][w], v[13][w]);
+        put(3, m);
+    } else {
+        uint32_t m[W] = {};
+        int kb = 0;
+#pragma unroll
+        for (int k = 0; k < kTcZpt; ++k) {
+#pragma unroll
+            for (int w = 0; w < W; ++w) m[w] = max3(m[w], v[k][w], v[k][w]);
+            if ((ends >> k) & 1u) {
+                put(kb++, m);
+#pragma unroll
+                for (int w = 0; w < W; ++w) m[w] = 0u;
+            }
+        }
+    }
+}
 constexpr float kIbFactor = 0.61685027506808491f;   // (pi/4)^2
 
 // P = PrecF32 is the split mode of FP32 plans: spectrum and taps are each
@@ -112,7 +177,12 @@ constexpr float kIbFactor = 0.61685027506808491f;   // (pi/4)^2
 // about 2^-16 of the product, is dropped), the template image is twice as
 // large (its lo half `b_lo` bytes after the hi one), two spectrum windows per
 // stage, two stages, and the plane is stored in FP32.
-template <class P, int kMode>
+//
+// kPool: also write the plane's maxima over boxes of 2 columns x one row block
+// (blocks of 3 to 5 rows of a chunk half, chunks[].ends), which the harmonic sum
+// by bounds reads: the cells are at hand here, and a separate pass over the
+// plane takes 247 us at 2^22 bins x 193 rows BF16 (see pool_kernel).
+template <class P, int kMode, bool kPool>
 __global__ void __launch_bounds__(kTcThreads, 1)
     correlate_tc_kernel(const unsigned char *__restrict__ spec_a,
                         const unsigned char *__restrict__ spec_lo,
@@ -121,8 +191,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         const float *__restrict__ inv_energy,
                         void *__restrict__ out, double2 *__restrict__ partials,
                         int64_t n_r, int win_bytes, int b_bytes_max, int nbuf,
-                        unsigned int *flags,
-                        float4 *__restrict__ edges FDAS_BC_PARAM) {
+                        unsigned int *flags, float4 *__restrict__ edges,
+                        uint32_t *__restrict__ pool FDAS_BC_PARAM) {
     constexpr bool kSplit = P::id == FDAS_FP32;
     constexpr int kStages = kSplit ? 2 : kTcStages;
     constexpr int kParts = kSplit ? 2 : 1;   // hi (+ lo) operand images
@@ -302,6 +372,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         int j = 0;
         float sc[kTcZpt];   // 1 / E'_z (power) or 1 / sqrt(E'_z) (complex, half bins)
         int zfirst = 0;     // first template of this warp's part of the chunk
+        unsigned ends = 0u;      // kPool: last templates of the part's row blocks
+        int blk0 = 0;            // and its first row block
         typename P::real *zrow = static_cast<typename P::real *>(out);
         typename P::cpx *zcrow = static_cast<typename P::cpx *>(out);
         float2 s1 = make_float2(0.f, 0.f), s2 = make_float2(0.f, 0.f);
@@ -329,6 +401,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 else
                     zrow = static_cast<typename P::real *>(out) + (int64_t)zb * n_r + 4 * row;
                 zfirst = zb;
+                if constexpr (kPool) {
+                    ends = chunks[c].ends[part];
+                    blk0 = chunks[c].blk0[part];
+                }
             }
             const int b = j & 1;
             const bool got = mbar_wait(&acc_full[b], (j >> 1) & 1);
@@ -399,7 +475,25 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         if (FDAS_IN_BOUNDS((int64_t)(zfirst + k) * 2 * n_r + t * (2 * kTcTile) + 8 * row,
                                            8, bc.lim[2] * 2 * n_r, kSiteTcPlaneStore))
                             *reinterpret_cast<uint4 *>(o + (int64_t)k * 2 * n_r) = u;
+                        if constexpr (kPool) {
+                            v[k][0] = u.x;
+                            v[k][1] = u.y;
+                            v[k][2] = u.z;
+                            v[k][3] = u.w;
+                        }
+                    } else if constexpr (kPool) {
+                        v[k][0] = v[k][1] = v[k][2] = v[k][3] = 0u;
                     }
+                }
+                if constexpr (kPool) {
+                    // 4 boxes per lane and row block (the half bin that lane 31
+                    // leaves joins its box in tc_ib_fixup_kernel)
+                    pool_blocks_of<4>(v, ends, [&](int kb, const uint32_t (&m)[4]) {
+                        const int64_t w = (int64_t)(blk0 + kb) * (n_r / 2) + t * (kTcTile / 2) + 2 * row;
+                        if (FDAS_IN_BOUNDS(w, 2, bc.lim[3], kSiteTcPlaneStore))
+                            *reinterpret_cast<uint2 *>(pool + w) =
+                                make_uint2(pool_pair<P>(m[0], m[1]), pool_pair<P>(m[2], m[3]));
+                    });
                 }
             } else if constexpr (kMode == kCplx) {
                 typename P::cpx *oc = zcrow + t * kTcTile;
@@ -434,23 +528,40 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 s1 = __fadd2_rn(s1, __fadd2_rn(p01, p23));
                 s2 = __ffma2_rn(p01, p01, s2);
                 s2 = __ffma2_rn(p23, p23, s2);
-                if (k < zvalid &&
-                    FDAS_IN_BOUNDS((int64_t)(zfirst + k) * n_r + t * kTcTile + 4 * row, 4,
-                                   bc.lim[2] * n_r, kSiteTcPlaneStore)) {
-                    if constexpr (kSplit) {
+                const bool in = k < zvalid &&
+                                FDAS_IN_BOUNDS((int64_t)(zfirst + k) * n_r + t * kTcTile + 4 * row, 4,
+                                               bc.lim[2] * n_r, kSiteTcPlaneStore);
+                if constexpr (kSplit) {
+                    if (in)
                         *reinterpret_cast<float4 *>(o + (int64_t)k * n_r) =
                             make_float4(p01.x, p01.y, p23.x, p23.y);
-                    } else {
-                        const typename P::cpx lo =
-                            P::st(ps == 1.f ? p01 : __fmul2_rn(p01, make_float2(ps, ps)));
-                        const typename P::cpx hi =
-                            P::st(ps == 1.f ? p23 : __fmul2_rn(p23, make_float2(ps, ps)));
-                        uint2 w;
-                        memcpy(&w.x, &lo, 4);
-                        memcpy(&w.y, &hi, 4);
-                        *reinterpret_cast<uint2 *>(o + (int64_t)k * n_r) = w;
+                    if constexpr (kPool) {
+                        // (columns past the part's templates are 0)
+                        v[k][0] = __float_as_uint(fmaxf(p01.x, p01.y));
+                        v[k][1] = __float_as_uint(fmaxf(p23.x, p23.y));
+                    }
+                } else {
+                    const typename P::cpx lo =
+                        P::st(ps == 1.f ? p01 : __fmul2_rn(p01, make_float2(ps, ps)));
+                    const typename P::cpx hi =
+                        P::st(ps == 1.f ? p23 : __fmul2_rn(p23, make_float2(ps, ps)));
+                    uint2 w;
+                    memcpy(&w.x, &lo, 4);
+                    memcpy(&w.y, &hi, 4);
+                    if (in) *reinterpret_cast<uint2 *>(o + (int64_t)k * n_r) = w;
+                    if constexpr (kPool) {
+                        v[k][0] = w.x;
+                        v[k][1] = w.y;
                     }
                 }
+            }
+            if constexpr (kPool) {
+                // two boxes per lane and row block
+                pool_blocks_of<2, kSplit>(v, ends, [&](int kb, const uint32_t (&m)[2]) {
+                    const int64_t w = (int64_t)(blk0 + kb) * (n_r / 4) + t * (kTcTile / 4) + row;
+                    if (FDAS_IN_BOUNDS(w, 1, bc.lim[3], kSiteTcPlaneStore))
+                        pool[w] = pool_pair<P>(m[0], m[1]);
+                });
             }
             }
             // FP32 within a tile, compensated FP32 across tiles
@@ -576,31 +687,45 @@ __global__ void tc_energy_kernel(float *__restrict__ inv_energy, const double *_
 // (z, tile, quarter) of the edge table holds that quarter's first F (lane 0,
 // .x .y) and last F (lane 31, .z .w); the half bin after the last F uses the
 // next entry's first F, or F(N_r) = 0 after the last tile.  One FP64 partial
-// (sum Q, sum Q^2) per CTA, after the tensor kernel's.
+// (sum Q, sum Q^2) per CTA, after the tensor kernel's.  A thread takes the rows
+// of one row block (blk; of one row without a pooled plane), so that it alone
+// raises the block's box there.
 template <class P>
 __global__ void __launch_bounds__(256)
     tc_ib_fixup_kernel(const float4 *__restrict__ edges, typename P::real *__restrict__ plane,
-                       double2 *__restrict__ partials, int64_t n_r, int n_z) {
+                       double2 *__restrict__ partials, int64_t n_r, int n_blk,
+                       const int32_t *__restrict__ blk, uint16_t *__restrict__ pool) {
     __shared__ double red[2][8];
     const int64_t n_tiles = n_r / kTcTile;
-    const int64_t n = (int64_t)n_z * n_tiles * 4;
+    const int64_t n = (int64_t)n_blk * n_tiles * 4;
     float s1 = 0.f, s2 = 0.f;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const int q = (int)(i & 3);
-        const int64_t zt = i >> 2;
-        const int64_t t = zt % n_tiles, z = zt / n_tiles;
-        const float4 a = edges[i];
-        float2 nx = make_float2(0.f, 0.f);
-        if (q < 3 || t + 1 < n_tiles) {
-            const float4 b = edges[i + 1];
-            nx = make_float2(b.x, b.y);
-        }
-        const float dr = a.z - nx.x, di = a.w - nx.y;
-        const float Q = kIbFactor * fmaf(dr, dr, di * di);
+        const int64_t t = (i >> 2) % n_tiles;
+        const int kb = (int)((i >> 2) / n_tiles);
+        const int z0 = pool != nullptr ? blk[kb] : kb, z1 = pool != nullptr ? blk[kb + 1] : kb + 1;
         const int64_t r = t * kTcTile + 128 * q + 127;
-        plane[z * 2 * n_r + 2 * r + 1] = P::str(Q * P::plane_scale);
-        s1 += Q;
-        s2 = fmaf(Q, Q, s2);
+        float top = 0.f;
+        for (int z = z0; z < z1; ++z) {
+            const int64_t e = ((int64_t)z * n_tiles + t) * 4 + q;
+            const float4 a = edges[e];
+            float2 nx = make_float2(0.f, 0.f);
+            if (q < 3 || t + 1 < n_tiles) {
+                const float4 b = edges[e + 1];
+                nx = make_float2(b.x, b.y);
+            }
+            const float dr = a.z - nx.x, di = a.w - nx.y;
+            const float Q = kIbFactor * fmaf(dr, dr, di * di);
+            const typename P::real h = P::str(Q * P::plane_scale);
+            plane[(int64_t)z * 2 * n_r + 2 * r + 1] = h;
+            top = fmaxf(top, P::ldr(h) * (1.0f / P::plane_scale));
+            s1 += Q;
+            s2 = fmaf(Q, Q, s2);
+        }
+        if (pool != nullptr) {
+            __half *box = reinterpret_cast<__half *>(pool) + (int64_t)kb * n_r + r;
+            *box = __hmax(*box, __float2half_rn(top));
+        }
     }
     double a1 = s1, a2 = s2;
 #pragma unroll
@@ -648,12 +773,15 @@ size_t tc_smem_bytes(int max_ks, int win, bool split, int nbuf) {
     return std::max(need, kTcMinSmem);
 }
 
-template <class P, int kMode>
+template <class P, int kMode, bool kPool = false>
 fdas_status launch_tc_P(Plan &p, const void *spec_padded, void *plane, double2 *partials,
-                        cudaStream_t s) {
+                        cudaStream_t s, uint16_t *pool = nullptr) {
+    if constexpr (!kPool && kMode != kCplx)
+        if (pool != nullptr)
+            return launch_tc_P<P, kMode, true>(p, spec_padded, plane, partials, s, pool);
     constexpr bool kSplit = P::id == FDAS_FP32;
     const size_t smem = tc_smem_bytes(p.tc_max_ks, p.tc_win, kSplit, p.tc_nbuf);
-    auto k = correlate_tc_kernel<P, kMode>;
+    auto k = correlate_tc_kernel<P, kMode, kPool>;
     FDAS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = correlate_tc_ctas(p);
     const void *spec_a = spec_padded, *spec_lo = nullptr;
@@ -673,12 +801,15 @@ fdas_status launch_tc_P(Plan &p, const void *spec_padded, void *plane, double2 *
                                       p.tc_n_ch,
                                       p.tc_inv_energy, plane, partials, p.n_r,
                                       p.tc_win * 4,
-                                      p.tc_max_ks * kTcSlab, p.tc_nbuf, p.flags, p.tc_edges
-                                      FDAS_BC_ARG(p.tc_img_bytes, 4 * p.spec_pad_elems, p.n_z));
+                                      p.tc_max_ks * kTcSlab, p.tc_nbuf, p.flags, p.tc_edges,
+                                      (uint32_t *)pool
+                                      FDAS_BC_ARG(p.tc_img_bytes, 4 * p.spec_pad_elems, p.n_z,
+                                                  (int64_t)p.pool_nb * plane_cols(p) / 4));
     FDAS_CUDA_TRY(cudaGetLastError());
     if constexpr (kMode == kInterbin) {
         tc_ib_fixup_kernel<P><<<tc_ib_fixup_ctas(p), 256, 0, s>>>(
-            p.tc_edges, (typename P::real *)plane, partials + grid, p.n_r, p.n_z);
+            p.tc_edges, (typename P::real *)plane, partials + grid, p.n_r,
+            pool != nullptr ? p.pool_nb : p.n_z, p.pool_blk, pool);
         FDAS_CUDA_TRY(cudaGetLastError());
     }
     return FDAS_OK;
@@ -726,6 +857,17 @@ std::vector<TcChunk> tc_chunk_table(const Plan &p, const std::vector<int32_t> &m
         c.kofs = (W0 - mc) & ~3;
         const int kc = (W0 - c.kofs + mc + 4 + 7) / 8 * 8;   // complex taps q in [0, kc)
         c.ks = kc / 8;
+        // row blocks of each half: runs of 3 or 4 rows (a half of 1, 2 or 5
+        // templates ends in a shorter one, at the edge of the plane)
+        for (int h = 0; h < 2; ++h) {
+            const int n = c.n_part[h], nb = (n + 3) / 4;
+            // (short blocks last there, else first)
+            const bool upper = n < kTcZpt && c.z_part[h] + n == p.n_z;
+            c.ends[h] = 0;
+            c.blk0[h] = 0;
+            for (int i = 1; i <= nb; ++i)
+                c.ends[h] |= (uint16_t)(1u << ((upper ? n - (nb - i) * n / nb : i * n / nb) - 1));
+        }
         c.b_off = b_off;
         b_off += (int64_t)c.ks * kTcSlab;
         wmax = std::max(wmax, c.kofs + kc);
@@ -735,6 +877,24 @@ std::vector<TcChunk> tc_chunk_table(const Plan &p, const std::vector<int32_t> &m
     *win = (4 * (kTcRows - 1) + wmax + 3) / 4 * 4;
     *max_ks = kmax;
     return out;
+}
+
+std::vector<int32_t> tc_pool_blocks(std::vector<TcChunk> &table, int n_z) {
+    std::vector<int32_t> first;
+    for (const TcChunk &c : table)
+        for (int h = 0; h < 2; ++h)
+            for (int k = 0, start = 0; k < c.n_part[h]; ++k)
+                if ((c.ends[h] >> k) & 1) {
+                    first.push_back(c.z_part[h] + start);
+                    start = k + 1;
+                }
+    std::sort(first.begin(), first.end());
+    for (TcChunk &c : table)
+        for (int h = 0; h < 2; ++h)
+            c.blk0[h] = (int32_t)(std::lower_bound(first.begin(), first.end(), c.z_part[h]) -
+                                  first.begin());
+    first.push_back(n_z);
+    return first;
 }
 
 bool tc_applicable(const Plan &p, std::string *why) {
@@ -818,20 +978,20 @@ fdas_status launch_tc_bank(Plan &p, cudaStream_t s) {
 }
 
 fdas_status launch_correlate_tc(Plan &p, const void *spec_padded, void *plane, double2 *partials,
-                                cudaStream_t s, bool cplx) {
+                                cudaStream_t s, bool cplx, uint16_t *pool) {
     switch (p.prec) {
         case FDAS_BF16:
             return cplx ? launch_tc_P<PrecBF16, kCplx>(p, spec_padded, plane, partials, s)
-                        : launch_tc_P<PrecBF16, kPower>(p, spec_padded, plane, partials, s);
+                        : launch_tc_P<PrecBF16, kPower>(p, spec_padded, plane, partials, s, pool);
         case FDAS_FP16:
             return cplx ? launch_tc_P<PrecF16, kCplx>(p, spec_padded, plane, partials, s)
-                        : launch_tc_P<PrecF16, kPower>(p, spec_padded, plane, partials, s);
+                        : launch_tc_P<PrecF16, kPower>(p, spec_padded, plane, partials, s, pool);
         case FDAS_FP32:
             if (cplx) {
                 set_error("the split tensor-core correlation writes power planes only");
                 return FDAS_ERR_UNSUPPORTED;
             }
-            return launch_tc_P<PrecF32, kPower>(p, spec_padded, plane, partials, s);
+            return launch_tc_P<PrecF32, kPower>(p, spec_padded, plane, partials, s, pool);
         default:
             set_error("tensor-core correlation: 16-bit precisions only");
             return FDAS_ERR_UNSUPPORTED;
@@ -839,14 +999,16 @@ fdas_status launch_correlate_tc(Plan &p, const void *spec_padded, void *plane, d
 }
 
 fdas_status launch_interbin_tc(Plan &p, const void *spec_padded, void *plane, double2 *partials,
-                               cudaStream_t s) {
+                               cudaStream_t s, uint16_t *pool) {
     if (!p.tc_edges) {
         set_error("tensor-core interbinning: the plan holds no edge table");
         return FDAS_ERR_UNSUPPORTED;
     }
     switch (p.prec) {
-        case FDAS_BF16: return launch_tc_P<PrecBF16, kInterbin>(p, spec_padded, plane, partials, s);
-        case FDAS_FP16: return launch_tc_P<PrecF16, kInterbin>(p, spec_padded, plane, partials, s);
+        case FDAS_BF16:
+            return launch_tc_P<PrecBF16, kInterbin>(p, spec_padded, plane, partials, s, pool);
+        case FDAS_FP16:
+            return launch_tc_P<PrecF16, kInterbin>(p, spec_padded, plane, partials, s, pool);
         default:
             set_error("tensor-core correlation: 16-bit precisions only");
             return FDAS_ERR_UNSUPPORTED;

@@ -154,6 +154,10 @@ struct TcChunk {
     int32_t kofs;      // first complex element of the window it reads (multiple of 4)
     int32_t ks;        // K steps of 8 complex taps (16 real elements)
     int64_t b_off;     // byte offset of the chunk's template image in tc_bank
+    // pooled plane: bit k of ends[h] marks the last template of a row block of
+    // half h, blk0[h] is the half's first row block
+    uint16_t ends[2];
+    int32_t blk0[2];
 };
 
 // ---------------------------------------------------------------------------
@@ -203,6 +207,7 @@ struct Plan {
     // of 2 bins x one row block, the blocks' first rows, and per block and
     // harmonic the source blocks
     bool pool_on = false;
+    int64_t pool_bytes = 0;
     int pool_nb = 0;
     uint16_t *pool[2] = {nullptr, nullptr};   // [pool_nb][plane_cols / 2] FP16
     int32_t *pool_blk = nullptr;              // [pool_nb + 1]
@@ -283,8 +288,10 @@ fdas_status launch_spectrum(Plan &p, const float *x, void *spec_out_padded,
                             float *medians, cudaStream_t s);
 // cplx: write the complex F (plane of the plan's complex type) instead of
 // |F|^2 and its statistics
+// (pool: also write the pooled plane; the tensor-core correlation only)
 fdas_status launch_correlate(Plan &p, const void *spec_padded, void *plane,
-                             double2 *partials, cudaStream_t s, bool cplx = false);
+                             double2 *partials, cudaStream_t s, bool cplx = false,
+                             uint16_t *pool = nullptr);
 int correlate_ctas(const Plan &p);
 // tensor-core correlation: whether it applies to the plan's geometry, the
 // host-side chunk table, the operand images (from the FP64 taps) and launch
@@ -294,12 +301,14 @@ std::vector<TcChunk> tc_chunk_table(const Plan &p, const std::vector<int32_t> &m
                                     int *max_ks);
 fdas_status launch_tc_bank(Plan &p, cudaStream_t s);
 fdas_status launch_correlate_tc(Plan &p, const void *spec_padded, void *plane, double2 *partials,
-                                cudaStream_t s, bool cplx);
+                                cudaStream_t s, bool cplx, uint16_t *pool = nullptr);
 int correlate_tc_ctas(const Plan &p);
+// first rows of the row blocks of a chunk table (and n_z); sets its blk0
+std::vector<int32_t> tc_pool_blocks(std::vector<TcChunk> &table, int n_z);
 // interbinning fused into the tensor-core epilogue: the half-bin plane and
 // its partials (interbin_tc_partials of them), using the plan's edge table
 fdas_status launch_interbin_tc(Plan &p, const void *spec_padded, void *plane, double2 *partials,
-                               cudaStream_t s);
+                               cudaStream_t s, uint16_t *pool = nullptr);
 int interbin_tc_partials(const Plan &p);
 int64_t tc_edge_bytes(const Plan &p);
 int64_t tc_bank_bytes(const std::vector<TcChunk> &table);
@@ -313,17 +322,19 @@ inline int64_t plane_cols(const Plan &p) { return p.interbin ? 2 * p.n_r : p.n_r
 fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partials,
                                   const double *given_stats, TrialStats *out,
                                   cudaStream_t s);
-// buf: which of the plan's two planes' workspaces the call may use
-fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf,
+// buf: which of the plan's two pooled planes the call may use; pooled: it
+// already holds this plane's maxima
+fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, bool pooled,
                                       const TrialStats *st, uint32_t rank,
                                       cudaStream_t s);
+bool sums_by_bounds(const Plan &p);   // whether launch_harmonic_threshold goes by bounds
 // the same crossings from bounds on boxes of cells (pool_on plans)
 constexpr int kPoolMaxRows = 4;   // rows of a block
 std::vector<int32_t> pool_blocks(int n_z);
 bool pool_sources(const std::vector<int32_t> &blk, int n_z, int iz0, int H,
                   std::vector<uint32_t> *src, std::vector<uint32_t> *masks);
-fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, const TrialStats *st,
-                                  uint32_t rank, cudaStream_t s);
+fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, bool pooled,
+                                  const TrialStats *st, uint32_t rank, cudaStream_t s);
 fdas_status launch_harmonic_sums(Plan &p, const void *plane, float *out,
                                  cudaStream_t s);
 fdas_status launch_stuck_wait(unsigned int *flags, long long limit_cycles, cudaStream_t s);

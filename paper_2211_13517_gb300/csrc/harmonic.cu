@@ -1045,10 +1045,12 @@ fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partia
     return FDAS_OK;
 }
 
-fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, const TrialStats *st,
-                                      uint32_t rank, cudaStream_t s) {
-    const bool by_bounds = p.pool_on && p.n_r >= kBoundMinCols;
-    if (by_bounds) FDAS_TRY(launch_harmonic_bound(p, plane, buf, st, rank, s));
+bool sums_by_bounds(const Plan &p) { return p.pool_on && p.n_r >= kBoundMinCols; }
+
+fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, bool pooled,
+                                      const TrialStats *st, uint32_t rank, cudaStream_t s) {
+    const bool by_bounds = sums_by_bounds(p);
+    if (by_bounds) FDAS_TRY(launch_harmonic_bound(p, plane, buf, pooled, st, rank, s));
     switch (p.prec) {
         case FDAS_FP32: return launch_hs_P<PrecF32, false>(p, plane, st, rank, nullptr, by_bounds, s);
         case FDAS_BF16: return launch_hs_P<PrecBF16, false>(p, plane, st, rank, nullptr, by_bounds, s);

@@ -40,7 +40,9 @@ namespace fdas {
 namespace {
 
 // ---------------------------------------------------------------------------
-// maxima of 2 bins x one row block, from a plane.  A thread reduces 8
+// maxima of 2 bins x one row block, from a plane (of the overlap-save
+// correlator, or a caller's; the tensor-core correlation writes its own).  A
+// thread reduces 8
 // consecutive bins of the block's rows (at most kPoolMaxRows; 16-byte loads,
 // all of them in flight).  Reads the plane once: HBM bound.
 // ---------------------------------------------------------------------------
@@ -517,12 +519,14 @@ fdas_status launch_bound(Plan &p, const void *plane, int buf, const TrialStats *
 }
 
 template <class P>
-fdas_status launch_bound_P(Plan &p, const void *plane, int buf, const TrialStats *st, uint32_t rank,
-                           cudaStream_t s) {
-    dim3 grid((unsigned)((p.n_r / 8 + 255) / 256), (unsigned)p.pool_nb);
-    pool_kernel<P><<<grid, 256, 0, s>>>((const typename P::real *)plane, p.pool[buf], p.pool_blk,
-                                        p.n_r);
-    FDAS_CUDA_TRY(cudaGetLastError());
+fdas_status launch_bound_P(Plan &p, const void *plane, int buf, bool pooled, const TrialStats *st,
+                           uint32_t rank, cudaStream_t s) {
+    if (!pooled) {
+        dim3 grid((unsigned)((p.n_r / 8 + 255) / 256), (unsigned)p.pool_nb);
+        pool_kernel<P><<<grid, 256, 0, s>>>((const typename P::real *)plane, p.pool[buf], p.pool_blk,
+                                            p.n_r);
+        FDAS_CUDA_TRY(cudaGetLastError());
+    }
     switch (p.H) {
         case 1: return launch_bound<P, 1>(p, plane, buf, st, rank, s);
         case 2: return launch_bound<P, 2>(p, plane, buf, st, rank, s);
@@ -567,12 +571,12 @@ bool pool_sources(const std::vector<int32_t> &blk, int n_z, int iz0, int H,
     return true;
 }
 
-fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, const TrialStats *st,
-                                  uint32_t rank, cudaStream_t s) {
+fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, bool pooled,
+                                  const TrialStats *st, uint32_t rank, cudaStream_t s) {
     switch (p.prec) {
-        case FDAS_FP32: return launch_bound_P<PrecF32>(p, plane, buf, st, rank, s);
-        case FDAS_BF16: return launch_bound_P<PrecBF16>(p, plane, buf, st, rank, s);
-        default: return launch_bound_P<PrecF16>(p, plane, buf, st, rank, s);
+        case FDAS_FP32: return launch_bound_P<PrecF32>(p, plane, buf, pooled, st, rank, s);
+        case FDAS_BF16: return launch_bound_P<PrecBF16>(p, plane, buf, pooled, st, rank, s);
+        default: return launch_bound_P<PrecF16>(p, plane, buf, pooled, st, rank, s);
     }
 }
 

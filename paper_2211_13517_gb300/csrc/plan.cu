@@ -186,6 +186,26 @@ static void dfree(Plan &p, void *ptr) {
     cudaFree(ptr);
 }
 
+static void free_pool(Plan &p) {
+    for (int b = 0; b < 2; ++b) {
+        dfree(p, p.pool[b]);
+        p.pool[b] = nullptr;
+    }
+    dfree(p, p.pool_blk);
+    dfree(p, p.pool_src);
+    dfree(p, p.pool_masks);
+    dfree(p, p.pool_list);
+    dfree(p, p.pool_listed);
+    p.pool_blk = nullptr;
+    p.pool_src = nullptr;
+    p.pool_masks = nullptr;
+    p.pool_list = nullptr;
+    p.pool_listed = nullptr;
+    p.ws_bytes -= p.pool_bytes;
+    p.pool_bytes = 0;
+    p.pool_on = false;
+}
+
 static void free_plan_memory(Plan *p) {
     dfree(*p, p->bank);
     dfree(*p, p->taps);
@@ -208,12 +228,7 @@ static void free_plan_memory(Plan *p) {
         if (p->ev_conv[b]) cudaEventDestroy(p->ev_conv[b]);
         if (p->ev_hsum[b]) cudaEventDestroy(p->ev_hsum[b]);
     }
-    for (int b = 0; b < 2; ++b) dfree(*p, p->pool[b]);
-    dfree(*p, p->pool_blk);
-    dfree(*p, p->pool_src);
-    dfree(*p, p->pool_masks);
-    dfree(*p, p->pool_list);
-    dfree(*p, p->pool_listed);
+    free_pool(*p);
     dfree(*p, p->stats);
     dfree(*p, p->rank_ids);
     dfree(*p, p->cand);
@@ -446,9 +461,10 @@ static void set_length(Plan &p, int64_t n) {
 // the correlation (and interbinning) of one series into `plane`, leaving
 // plane_partials(v) FP64 partials in `partials`
 static fdas_status launch_plane(Plan &v, const void *spec_pad, void *plane, double2 *partials,
-                                cudaStream_t s) {
-    if (!v.interbin) return launch_correlate(v, spec_pad, plane, partials, s);
-    if (v.correlator == FDAS_CORR_TENSOR) return launch_interbin_tc(v, spec_pad, plane, partials, s);
+                                cudaStream_t s, uint16_t *pool = nullptr) {
+    if (!v.interbin) return launch_correlate(v, spec_pad, plane, partials, s, false, pool);
+    if (v.correlator == FDAS_CORR_TENSOR)
+        return launch_interbin_tc(v, spec_pad, plane, partials, s, pool);
     FDAS_TRY(launch_correlate(v, spec_pad, v.corr, partials, s, true));
     return launch_interbin(v, v.corr, plane, partials, s);
 }
@@ -488,6 +504,31 @@ static bool bounds_pay(const Plan &p) {
     return p.harm_mode == FDAS_HARM_TOP && p.H >= 2 && p.H <= 16 && p.n_z >= 12 &&
            p.norm_mode == FDAS_NORM_MEDIAN && p.thr_mode == FDAS_THRESH_GAMMA_TAIL &&
            p.sigma >= (p.H == 16 ? 5.4 : 5.0);
+}
+
+// the workspace of the sums by bounds for these row blocks (none where they
+// do not pay or a harmonic's sources span more than two blocks)
+static fdas_status build_pool(Plan &p, const std::vector<int32_t> &blk) {
+    std::vector<uint32_t> src, masks;
+    if (!bounds_pay(p) || !pool_sources(blk, p.n_z, p.iz0, p.H, &src, &masks)) return FDAS_OK;
+    const int64_t before = p.ws_bytes;
+    p.pool_nb = (int)blk.size() - 1;
+    const int64_t boxes = (int64_t)p.pool_nb * (plane_cols(p) / 2);
+    p.pool_list_cap = (unsigned)std::max<int64_t>(4096, boxes / 64);
+    for (int b = 0; b < 2; ++b)
+        FDAS_TRY(dalloc(p, &p.pool[b], sizeof(uint16_t) * (size_t)boxes, b == 0 ? "pool[0]" : "pool[1]"));
+    FDAS_TRY(dalloc(p, &p.pool_list, sizeof(unsigned long long) * p.pool_list_cap, "pool_list"));
+    FDAS_TRY(dalloc(p, &p.pool_listed, sizeof(unsigned int), "pool_listed"));
+    FDAS_TRY(dalloc(p, &p.pool_blk, sizeof(int32_t) * blk.size(), "pool_blk"));
+    FDAS_TRY(dalloc(p, &p.pool_src, sizeof(uint32_t) * src.size(), "pool_src"));
+    FDAS_TRY(dalloc(p, &p.pool_masks, sizeof(uint32_t) * masks.size(), "pool_masks"));
+    FDAS_CUDA_TRY(cudaMemcpy(p.pool_blk, blk.data(), sizeof(int32_t) * blk.size(), cudaMemcpyHostToDevice));
+    FDAS_CUDA_TRY(cudaMemcpy(p.pool_src, src.data(), sizeof(uint32_t) * src.size(), cudaMemcpyHostToDevice));
+    FDAS_CUDA_TRY(cudaMemcpy(p.pool_masks, masks.data(), sizeof(uint32_t) * masks.size(),
+                             cudaMemcpyHostToDevice));
+    p.pool_bytes = p.ws_bytes - before;
+    p.pool_on = true;
+    return FDAS_OK;
 }
 
 static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_max, double z_step,
@@ -680,30 +721,7 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
     // itself and needs only its edge table (allocated below)
     if (p.interbin && p.correlator != FDAS_CORR_TENSOR)
         PLAN_TRY(dalloc(p, &p.corr, cb * (size_t)p.n_z * (size_t)p.n_r, "corr"));
-    {
-        std::vector<uint32_t> src, masks;
-        const std::vector<int32_t> blk = pool_blocks(p.n_z);
-        p.pool_on = bounds_pay(p) && pool_sources(blk, p.n_z, p.iz0, p.H, &src, &masks);
-        if (p.pool_on) {
-            p.pool_nb = (int)blk.size() - 1;
-            const int64_t boxes = (int64_t)p.pool_nb * (plane_cols(p) / 2);
-            p.pool_list_cap = (unsigned)std::max<int64_t>(4096, boxes / 64);
-            for (int b = 0; b < 2; ++b)
-                PLAN_TRY(dalloc(p, &p.pool[b], sizeof(uint16_t) * (size_t)boxes,
-                                b == 0 ? "pool[0]" : "pool[1]"));
-            PLAN_TRY(dalloc(p, &p.pool_list, sizeof(unsigned long long) * p.pool_list_cap, "pool_list"));
-            PLAN_TRY(dalloc(p, &p.pool_listed, sizeof(unsigned int), "pool_listed"));
-            PLAN_TRY(dalloc(p, &p.pool_blk, sizeof(int32_t) * blk.size(), "pool_blk"));
-            PLAN_TRY(dalloc(p, &p.pool_src, sizeof(uint32_t) * src.size(), "pool_src"));
-            PLAN_TRY(dalloc(p, &p.pool_masks, sizeof(uint32_t) * masks.size(), "pool_masks"));
-            PLAN_CUDA(cudaMemcpy(p.pool_masks, masks.data(), sizeof(uint32_t) * masks.size(),
-                                 cudaMemcpyHostToDevice));
-            PLAN_CUDA(cudaMemcpy(p.pool_blk, blk.data(), sizeof(int32_t) * blk.size(),
-                                 cudaMemcpyHostToDevice));
-            PLAN_CUDA(cudaMemcpy(p.pool_src, src.data(), sizeof(uint32_t) * src.size(),
-                                 cudaMemcpyHostToDevice));
-        }
-    }
+    PLAN_TRY(build_pool(p, tc_table.empty() ? pool_blocks(p.n_z) : tc_pool_blocks(tc_table, p.n_z)));
     PLAN_TRY(grow_stats(p, 64));
     const int64_t rec_cap = next_pow2(p.max_cands);
     PLAN_TRY(dalloc(p, &p.cand, sizeof(CandRec) * (size_t)rec_cap, "cand"));
@@ -1029,7 +1047,10 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
             FDAS_CUDA_TRY(cudaStreamWaitEvent(s, p.ev_hsum[b], 0));
             if (p.profiling) e1 = mark(s);
         }
-        FDAS_TRY(launch_plane(v, p.spec_pad, p.plane[b], p.partials[b], s));
+        Plan hv = harm_view(v);
+        const bool pooled = sums_by_bounds(hv) && v.correlator == FDAS_CORR_TENSOR;
+        FDAS_TRY(launch_plane(v, p.spec_pad, p.plane[b], p.partials[b], s,
+                              pooled ? p.pool[b] : nullptr));
 #ifdef FDAS_CHECK_BOUNDS
         if (p.plant_canary && t == 0) {
             // FDAS_FAULT=canary: one byte of the guard after the plane
@@ -1044,9 +1065,8 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
         FDAS_CUDA_TRY(cudaStreamWaitEvent(hs, p.ev_conv[b], 0));
         cudaEvent_t e3 = p.profiling ? mark(hs) : nullptr;
         TrialStats *ts = p.stats + rank[t];
-        Plan hv = harm_view(v);
         FDAS_TRY(launch_finalize_stats(hv, p.partials[b], plane_partials(v), nullptr, ts, hs));
-        FDAS_TRY(launch_harmonic_threshold(hv, p.plane[b], b, ts, (uint32_t)rank[t], hs));
+        FDAS_TRY(launch_harmonic_threshold(hv, p.plane[b], b, pooled, ts, (uint32_t)rank[t], hs));
         FDAS_DEBUG_CHECK(p, hs, "the harmonic sum of series " + std::to_string(t));
         cudaEvent_t e4 = p.profiling ? mark(hs) : nullptr;
         FDAS_CUDA_TRY(cudaEventRecord(p.ev_hsum[b], hs));
@@ -1282,6 +1302,8 @@ static fdas_status retable_tc(Plan &p, int order) {
         return FDAS_ERR_UNSUPPORTED;
     }
     FDAS_CUDA_TRY(cudaDeviceSynchronize());
+    free_pool(p);   // its row blocks follow the chunks
+    FDAS_TRY(build_pool(p, tc_pool_blocks(table, p.n_z)));
     const int64_t img = tc_bank_bytes(table);
     p.ws_bytes -= p.tc_img_bytes + (int64_t)sizeof(TcChunk) * old_n;
     dfree(p, p.tc_chunks);
@@ -1567,7 +1589,7 @@ fdas_status fdas_threshold(fdas_plan *plan, const void *plane, const double *sta
     FDAS_CUDA_TRY(cudaMemsetAsync(p.flags, 0, sizeof(unsigned int), s));
     Plan hv = harm_view(p);
     FDAS_TRY(launch_finalize_stats(hv, nullptr, 0, stats, p.stats, s));
-    FDAS_TRY(launch_harmonic_threshold(hv, plane, 0, p.stats, 0, s));
+    FDAS_TRY(launch_harmonic_threshold(hv, plane, 0, false, p.stats, 0, s));
     const fdas_status st = collect(p, cands, capacity, n_found, s);
     FDAS_DEBUG_CHECK(p, s, "fdas_threshold");
     return st;
