@@ -291,7 +291,8 @@ fdas_status fdas_search_async(fdas_plan *plan, const fdas_series *batch,
  *   F(r, z) = sum_{e=-m..m} X_{k0+e} conj(rho(delta - e, z)),   P = |F|^2,
  * rho the unnormalised response above (so a signal c rho(r0 - k, z0) gives
  * P(r0, z0) ~ |c|^2 at any z0), bins outside [0, N_r) counted as 0.  The
- * integrals are Gauss-Legendre sums with 512 nodes, FP32 arithmetic.  The
+ * integrals are Gauss-Legendre sums with 512 nodes (in the gradient with
+ * respect to the spectrum 128, 256 or 512, as |z| needs), FP32 arithmetic.  The
  * window is held fixed when differentiating.
  * `spectrum` is always FP32 complex (N_r float pairs, device), e.g. the
  * output of fdas_spectrum on an FP32 plan.

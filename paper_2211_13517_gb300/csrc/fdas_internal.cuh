@@ -248,6 +248,7 @@ struct Plan {
     cudaEvent_t ev_start = nullptr;         // orders the copy stream after the caller's
     unsigned long long *host_small = nullptr;  // pinned: {count, flags}
     float2 *gl_nodes = nullptr;     // Gauss-Legendre (u, w) on [0, 1] for P(r, z)
+    float4 *gl_fine = nullptr;      // (u, low part of u, w) of the rules of 512, 256, 128 nodes
     fdas_seed *ref_seeds = nullptr;        // device staging of refine seeds
     fdas_refined *ref_out = nullptr;       // device staging of refine results
     int64_t ref_cap = 0;
@@ -345,7 +346,7 @@ fdas_status launch_candidates_finish(Plan &p, int64_t n, fdas_candidate *out_dev
 // from the count in device memory
 fdas_status launch_candidates_finish_async(Plan &p, int64_t capacity, unsigned int extra_flags,
                                            fdas_candidate *out_dev, cudaStream_t s);
-std::vector<float2> gauss_legendre_01(int n);
+const std::vector<float4> &refine_rules();   // refine_nodes(), half and a quarter of them
 int refine_nodes();
 fdas_status launch_fourier_power(Plan &p, const float2 *X, const double2 *rz, int n, float *power,
                                  float2 *grad, cudaStream_t s);

@@ -245,6 +245,7 @@ static void free_plan_memory(Plan *p) {
     if (p->cpy) cudaStreamDestroy(p->cpy);
     if (p->ev_start) cudaEventDestroy(p->ev_start);
     dfree(*p, p->gl_nodes);
+    dfree(*p, p->gl_fine);
     dfree(*p, p->ref_seeds);
     dfree(*p, p->ref_out);
     if (p->host_small) cudaFreeHost(p->host_small);
@@ -759,7 +760,12 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
     }
 
     {
-        const std::vector<float2> gl = gauss_legendre_01(refine_nodes());
+        const std::vector<float4> &fine = refine_rules();
+        std::vector<float2> gl;   // the forward sums take the first rule, rounded
+        for (int i = 0; i < refine_nodes(); ++i) gl.push_back(make_float2(fine[i].x, fine[i].z));
+        PLAN_TRY(dalloc(p, &p.gl_fine, sizeof(float4) * fine.size(), "gl_fine"));
+        PLAN_CUDA(cudaMemcpy(p.gl_fine, fine.data(), sizeof(float4) * fine.size(),
+                             cudaMemcpyHostToDevice));
         PLAN_TRY(dalloc(p, &p.gl_nodes, sizeof(float2) * gl.size(), "gl_nodes"));
         PLAN_CUDA(cudaMemcpy(p.gl_nodes, gl.data(), sizeof(float2) * gl.size(),
                              cudaMemcpyHostToDevice));
