@@ -247,6 +247,7 @@ struct Plan {
     cudaEvent_t ev_consumed[2] = {nullptr, nullptr};
     cudaEvent_t ev_start = nullptr;         // orders the copy stream after the caller's
     unsigned long long *host_small = nullptr;  // pinned: {count, flags}
+    fdas_candidate *host_cands = nullptr;      // pinned: the first records of a search
     float2 *gl_nodes = nullptr;     // Gauss-Legendre (u, w) on [0, 1] for P(r, z)
     float4 *gl_fine = nullptr;      // (u, low part of u, w) of the rules of 512, 256, 128 nodes
     fdas_seed *ref_seeds = nullptr;        // device staging of refine seeds
@@ -339,6 +340,12 @@ fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, bool pool
 fdas_status launch_harmonic_sums(Plan &p, const void *plane, float *out,
                                  cudaStream_t s);
 fdas_status launch_stuck_wait(unsigned int *flags, long long limit_cycles, cudaStream_t s);
+// up to candidates_order_max() records ordered and converted into out_dev, from
+// the count in device memory; the count, the flags and the first `eager`
+// records also into the plan's page-locked host memory
+fdas_status launch_candidates_order(Plan &p, fdas_candidate *out_dev, int64_t eager, cudaStream_t s);
+fdas_status launch_init_search(Plan &p, const uint32_t *ids, int n, cudaStream_t s);
+int64_t candidates_order_max();
 fdas_status launch_candidates_finish(Plan &p, int64_t n, fdas_candidate *out_dev,
                                      cudaStream_t s);
 // stream-ordered end of a search: status and counts into p.async_res, the

@@ -40,8 +40,8 @@ struct ThrParams {
 __global__ void finalize_stats_kernel(const double2 *__restrict__ partials, int n_partials,
                                       const double *__restrict__ given, TrialStats *out,
                                       ThrParams tp, unsigned int *listed) {
-    __shared__ double sa[256], sb[256];
-    const int tid = threadIdx.x;
+    __shared__ double sa[8], sb[8];
+    const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0 && listed != nullptr) *listed = 0u;   // boxes of the bound sums that follow
     double a = 0.0, b = 0.0;
     if (given == nullptr) {
@@ -49,39 +49,43 @@ __global__ void finalize_stats_kernel(const double2 *__restrict__ partials, int 
             a += partials[i].x;
             b += partials[i].y;
         }
-    }
-    sa[tid] = a;
-    sb[tid] = b;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (tid < w) {
-            sa[tid] += sa[tid + w];
-            sb[tid] += sb[tid + w];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, off);
+            b += __shfl_xor_sync(0xffffffffu, b, off);
+        }
+        if (lane == 0) {
+            sa[tid >> 5] = a;
+            sb[tid >> 5] = b;
         }
         __syncthreads();
     }
-    if (tid == 0) {
-        double mean, sd;
-        if (given != nullptr) {
-            mean = given[0];
-            sd = given[1];
-        } else {
-            mean = sa[0] / tp.n_cells;
-            const double var = sb[0] / tp.n_cells - mean * mean;
-            sd = sqrt(var > 0.0 ? var : 0.0);
+    if (tid >= 8) return;   // one thread per threshold
+    double mean, sd;
+    if (given != nullptr) {
+        mean = given[0];
+        sd = given[1];
+    } else {
+        a = b = 0.0;
+        for (int w = 0; w < 8; ++w) {
+            a += sa[w];
+            b += sb[w];
         }
+        mean = a / tp.n_cells;
+        const double var = b / tp.n_cells - mean * mean;
+        sd = sqrt(var > 0.0 ? var : 0.0);
+    }
+    if (tid == 0) {
         out->mean = mean;
         out->std = sd;
-        for (int s = 0; s < 8; ++s) {
-            float t = 0.f;
-            if (s < tp.n_stages) {
-                const double h = (double)(1 << s);
-                t = tp.mode == FDAS_THRESH_GAMMA_TAIL ? (float)(mean * tp.G[s])
-                                                     : (float)(h * mean + tp.sigma * sqrt(h) * sd);
-            }
-            out->thr[s] = t;
-        }
     }
+    float t = 0.f;
+    if (tid < tp.n_stages) {
+        const double h = (double)(1 << tid);
+        t = tp.mode == FDAS_THRESH_GAMMA_TAIL ? (float)(mean * tp.G[tid])
+                                             : (float)(h * mean + tp.sigma * sqrt(h) * sd);
+    }
+    out->thr[tid] = t;
 }
 
 // ---------------------------------------------------------------------------
@@ -721,20 +725,31 @@ __global__ void collect_status_kernel(const unsigned long long *__restrict__ cou
     *out = r;
 }
 
-// log Q(h, x) for integer h: Q = exp(-x) sum_{k<h} x^k / k!
+// log Q(h, x), h a power of two up to 32: Q = exp(-x) sum_{k<h} x^k / k!, the sum
+// by Horner's rule (two FP64 functions in all; a logarithm and an exponential per
+// term took a chain of 2 h of them on a GPU with few FP64 lanes)
+__constant__ double kInv[32] = {0.0,      1.0,      1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,
+                                1.0 / 7,  1.0 / 8,  1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13,
+                                1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18, 1.0 / 19, 1.0 / 20,
+                                1.0 / 21, 1.0 / 22, 1.0 / 23, 1.0 / 24, 1.0 / 25, 1.0 / 26, 1.0 / 27,
+                                1.0 / 28, 1.0 / 29, 1.0 / 30, 1.0 / 31};
 __device__ double log_gamma_tail(int h, double x) {
     if (x <= 0.0) return 0.0;
-    const double lx = log(x);
-    double lt[32];
-    double mx = -1e300, lf = 0.0;
-    for (int k = 0; k < h; ++k) {
-        if (k > 0) lf += log((double)k);
-        lt[k] = k * lx - lf;
-        mx = fmax(mx, lt[k]);
+    if (x < 1e6) {   // x^31 / 31! stays far inside the range
+        double s = 1.0;
+        for (int k = h - 1; k > 0; --k) s = fma(s, x * kInv[k], 1.0);
+        return -x + log(s);
     }
-    double s = 0.0;
-    for (int k = 0; k < h; ++k) s += exp(lt[k] - mx);
-    return -x + mx + log(s);
+    // from the last term down: x^(h-1)/(h-1)! (1 + (h-1)/x (1 + (h-2)/x (...)))
+    const double lf = h <= 2 ? 0.0                     // log((h - 1)!)
+                      : h == 4  ? 1.791759469228055
+                      : h == 8  ? 8.525161361065415
+                      : h == 16 ? 27.899271383840894
+                                : 78.09222355331532;
+    const double y = 1.0 / x;
+    double t = 1.0;
+    for (int k = 1; k < h; ++k) t = fma(t, k * y, 1.0);
+    return -x + (h - 1) * log(x) - lf + log(t);
 }
 
 // Gaussian-equivalent sigma of an upper-tail probability given as log p
@@ -757,6 +772,26 @@ __device__ double sigma_from_logp(double lp) {
     return s;
 }
 
+// a crossing's Gaussian-equivalent significance
+__device__ __forceinline__ double sigma_of(const CandRec &c, const TrialStats &t, int mode) {
+    const int h = 1 << (int)((c.key >> 39) & 7);
+    if (mode == FDAS_THRESH_GAMMA_TAIL)
+        return sigma_from_logp(log_gamma_tail(h, (double)c.power / t.mean));
+    return ((double)c.power - h * t.mean) / (sqrt((double)h) * t.std);
+}
+
+__device__ __forceinline__ fdas_candidate candidate_of(const CandRec &c, uint32_t trial_id,
+                                                       double sig) {
+    fdas_candidate o;
+    o.trial_id = trial_id;
+    o.ir = (uint32_t)(c.key & 0x7fffff);
+    o.iz = (uint16_t)((c.key >> 23) & 0xffff);
+    o.harm = (uint16_t)(1 << (int)((c.key >> 39) & 7));
+    o.power = c.power;
+    o.sigma = (float)sig;
+    return o;
+}
+
 // records [0, n) (n = *n_dev when n_dev is set) into caller records; a
 // record whose batch rank is not below n_ranks (never one the harmonic
 // kernels wrote) is not read further
@@ -770,24 +805,66 @@ __global__ void finish_kernel(const CandRec *__restrict__ rec, int64_t n_host,
     const CandRec c = rec[i];
     const uint32_t rank = (uint32_t)(c.key >> 42);
     if ((int64_t)rank >= n_ranks) return;
-    const int s = (int)((c.key >> 39) & 7);
-    const int iz = (int)((c.key >> 23) & 0xffff);
-    const uint32_t ir = (uint32_t)(c.key & 0x7fffff);
-    const int h = 1 << s;
-    const TrialStats t = st[rank];
-    double sig;
-    if (mode == FDAS_THRESH_GAMMA_TAIL)
-        sig = sigma_from_logp(log_gamma_tail(h, (double)c.power / t.mean));
-    else
-        sig = ((double)c.power - h * t.mean) / (sqrt((double)h) * t.std);
-    fdas_candidate o;
-    o.trial_id = ids[rank];
-    o.ir = ir;
-    o.iz = (uint16_t)iz;
-    o.harm = (uint16_t)h;
-    o.power = c.power;
-    o.sigma = (float)sig;
-    out[i] = o;
+    out[i] = candidate_of(c, ids[rank], sigma_of(c, st[rank], mode));
+}
+
+// Ordering and conversion of up to kOrderMax records in one kernel, from the
+// count in device memory (only the count and the flags are reported for more
+// records, a full store or an error flag).  A record's place is the number of
+// smaller keys (keys are distinct): a warp counts for 8 records at a time, its
+// lanes over the keys; then 32 lanes convert 32 records.  The first `eager`
+// records and the outcome also go to page-locked host memory, which saves the
+// caller the copies.  Bound: latency, half of it FP64 functions.  The sort network
+// and finish_kernel, which larger lists take, are a chain of steps on one CTA
+// before they convert: 1234 records 46 + 40 us there, 13 here.
+constexpr int kOrderMax = 8192;
+constexpr int kOrderThreads = 128;
+__global__ void __launch_bounds__(kOrderThreads)
+    order_kernel(const CandRec *__restrict__ rec, const unsigned long long *__restrict__ count,
+                 const unsigned int *__restrict__ flags, int64_t store_cap,
+                 const TrialStats *__restrict__ st, const uint32_t *__restrict__ ids,
+                 int64_t n_ranks, fdas_candidate *__restrict__ out, int mode, int64_t eager,
+                 fdas_candidate *__restrict__ host_out, unsigned long long *__restrict__ host_res) {
+    __shared__ int place[32];
+    const unsigned long long total = *count;
+    const unsigned int fl = *flags;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        host_res[0] = total;
+        host_res[1] = fl;
+    }
+    if (total > (unsigned long long)kOrderMax || (int64_t)total > store_cap || (fl & 3u) != 0u) return;
+    const int n = (int)total, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int base = 32 * (int)blockIdx.x; base < n; base += 32 * (int)gridDim.x) {
+        unsigned long long key[8];
+        int less[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            key[r] = rec[min(base + 8 * warp + r, n - 1)].key;
+            less[r] = 0;
+        }
+        for (int j = lane; j < n; j += 32) {
+            const unsigned long long k = rec[j].key;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) less[r] += k < key[r];
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            less[r] = __reduce_add_sync(0xffffffffu, less[r]);
+            if (lane == 0) place[8 * warp + r] = less[r];
+        }
+        __syncthreads();
+        if (warp == 0 && base + lane < n) {
+            const CandRec c = rec[base + lane];
+            const uint32_t rank = (uint32_t)(c.key >> 42);
+            if ((int64_t)rank < n_ranks) {
+                const int at = place[lane];
+                const fdas_candidate o = candidate_of(c, ids[rank], sigma_of(c, st[rank], mode));
+                out[at] = o;
+                if (at < eager) host_out[at] = o;
+            }
+        }
+        __syncthreads();
+    }
 }
 
 template <class P, int H, bool kWriteSums, bool kGated>
@@ -1095,6 +1172,47 @@ static fdas_status launch_sort(Plan &p, int64_t n, const int64_t *n_dev, int64_t
     }
     return FDAS_OK;
 }
+
+fdas_status launch_candidates_order(Plan &p, fdas_candidate *out_dev, int64_t eager, cudaStream_t s) {
+    order_kernel<<<256, kOrderThreads, 0, s>>>(p.cand, p.cand_count, p.flags, p.store_cap, p.stats,
+                                               p.rank_ids, p.stats_cap, out_dev, p.thr_mode, eager,
+                                               p.host_cands, p.host_small);
+    FDAS_CUDA_TRY(cudaGetLastError());
+    p.launches[FDAS_PROF_FINISH] += 1;
+    return FDAS_OK;
+}
+
+// the counters of a search reset and, for up to kInitIds series, the trial ids
+// set from the launch's arguments (one launch instead of a copy and two fills)
+struct InitIds {
+    uint32_t id[32];
+};
+__global__ void init_search_kernel(InitIds ids, int n, uint32_t *__restrict__ rank_ids,
+                                   unsigned long long *__restrict__ count,
+                                   unsigned int *__restrict__ flags) {
+    const int t = threadIdx.x;
+    if (t < n) rank_ids[t] = ids.id[t];
+    if (t == 0) {
+        *count = 0ull;
+        *flags = 0u;
+    }
+}
+
+fdas_status launch_init_search(Plan &p, const uint32_t *ids, int n, cudaStream_t s) {
+    InitIds arg{};
+    if (n <= 32) {
+        for (int i = 0; i < n; ++i) arg.id[i] = ids[i];
+    } else {
+        // (a copy from pageable memory returns once the source has been read)
+        FDAS_CUDA_TRY(cudaMemcpyAsync(p.rank_ids, ids, sizeof(uint32_t) * (size_t)n,
+                                      cudaMemcpyHostToDevice, s));
+    }
+    init_search_kernel<<<1, 32, 0, s>>>(arg, n <= 32 ? n : 0, p.rank_ids, p.cand_count, p.flags);
+    FDAS_CUDA_TRY(cudaGetLastError());
+    return FDAS_OK;
+}
+
+int64_t candidates_order_max() { return kOrderMax; }
 
 fdas_status launch_candidates_finish(Plan &p, int64_t n, fdas_candidate *out_dev, cudaStream_t s) {
     if (n <= 0) return FDAS_OK;

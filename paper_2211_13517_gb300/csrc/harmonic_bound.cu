@@ -511,7 +511,8 @@ fdas_status launch_bound(Plan &p, const void *plane, int buf, const TrialStats *
     k<<<grid, 32, smem, s>>>(p.pool[buf], p.n_r, p.pool_nb, walk, p.pool_src, p.pool_masks, st,
                              p.pool_list, p.pool_list_cap, p.pool_listed, p.flags);
     FDAS_CUDA_TRY(cudaGetLastError());
-    harmonic_exact_kernel<P, H><<<kExactCtas * p.n_sms, kExactThreads, 0, s>>>(
+    const unsigned exact_ctas = std::min(kExactCtas * (unsigned)p.n_sms, p.pool_list_cap / 16);
+    harmonic_exact_kernel<P, H><<<exact_ctas, kExactThreads, 0, s>>>(
         p.pool_list, p.pool_list_cap, p.pool_listed, (const typename P::real *)plane, p.n_r, p.n_z,
         p.iz0, p.pool_blk, st, rank, p.cand, p.cand_count, p.store_cap);
     FDAS_CUDA_TRY(cudaGetLastError());

@@ -16,6 +16,8 @@ namespace fdas {
 
 static thread_local std::string g_last_error;
 
+constexpr int64_t kEagerCands = 2048;   // records copied to the host along with the count
+
 void set_error(const std::string &msg) { g_last_error = msg; }
 
 fdas_status cuda_status(cudaError_t e, const char *what) {
@@ -249,6 +251,7 @@ static void free_plan_memory(Plan *p) {
     dfree(*p, p->ref_seeds);
     dfree(*p, p->ref_out);
     if (p->host_small) cudaFreeHost(p->host_small);
+    if (p->host_cands) cudaFreeHost(p->host_cands);
     for (cudaEvent_t e : p->pools->events) cudaEventDestroy(e);
     if (p->aux) cudaStreamDestroy(p->aux);
     if (p->hi) cudaStreamDestroy(p->hi);
@@ -745,6 +748,7 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
         PLAN_CUDA(cudaEventCreateWithFlags(&p.ev_consumed[b], cudaEventDisableTiming));
     }
     PLAN_CUDA(cudaMallocHost((void **)&p.host_small, 4 * sizeof(unsigned long long)));
+    PLAN_CUDA(cudaMallocHost((void **)&p.host_cands, sizeof(fdas_candidate) * kEagerCands));
     // the harmonic sum of one series runs on the lowest-priority stream
     // beside the spectrum and correlation of the next on the highest: as the
     // harmonic sum's CTAs retire, the block scheduler places the correlation's
@@ -826,13 +830,16 @@ static bool is_device_ptr(const void *ptr) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// sort/convert the stored candidates and copy them out; blocking
+// Sort/convert the stored candidates and copy them out; blocking.  The
+// records of a search that found no more than order_kernel takes are in order
+// by the time the count is known, and for a host buffer the first kEagerCands
+// of them come with the count: one synchronisation instead of two.
 static fdas_status collect(Plan &p, fdas_candidate *cands, int64_t capacity, int64_t *n_found,
                            cudaStream_t s) {
-    FDAS_CUDA_TRY(cudaMemcpyAsync(p.host_small, p.cand_count, sizeof(unsigned long long),
-                                  cudaMemcpyDeviceToHost, s));
-    FDAS_CUDA_TRY(cudaMemcpyAsync(p.host_small + 1, p.flags, sizeof(unsigned int),
-                                  cudaMemcpyDeviceToHost, s));
+    const int64_t eager = capacity > 0 && !is_device_ptr(cands)
+                              ? std::min({capacity, (int64_t)kEagerCands, p.max_cands})
+                              : 0;
+    FDAS_TRY(launch_candidates_order(p, p.out_stage, eager, s));
     FDAS_CUDA_TRY(cudaStreamSynchronize(s));
     const int64_t total = (int64_t)p.host_small[0];
     unsigned int flags = (unsigned int)(p.host_small[1] & 0xffffffffu);
@@ -856,13 +863,19 @@ static fdas_status collect(Plan &p, fdas_candidate *cands, int64_t capacity, int
                   " (raise max_candidates or the threshold)");
         return FDAS_ERR_CAND_STORE_FULL;
     }
-    const int64_t stored = total;
-    FDAS_TRY(launch_candidates_finish(p, stored, p.out_stage, s));
-    const int64_t n_copy = std::min(stored, capacity);
-    if (n_copy > 0)
-        FDAS_CUDA_TRY(cudaMemcpyAsync(cands, p.out_stage, sizeof(fdas_candidate) * (size_t)n_copy,
+    const int64_t n_copy = std::min(total, capacity);
+    int64_t done = 0;   // records in the caller's buffer
+    if (total > candidates_order_max()) {
+        FDAS_TRY(launch_candidates_finish(p, total, p.out_stage, s));
+    } else if (eager > 0) {
+        done = std::min(n_copy, eager);
+        std::memcpy(cands, p.host_cands, sizeof(fdas_candidate) * (size_t)done);
+    }
+    if (n_copy > done)
+        FDAS_CUDA_TRY(cudaMemcpyAsync(cands + done, p.out_stage + done,
+                                      sizeof(fdas_candidate) * (size_t)(n_copy - done),
                                       cudaMemcpyDefault, s));
-    FDAS_CUDA_TRY(cudaStreamSynchronize(s));
+    if (n_copy > done || total > candidates_order_max()) FDAS_CUDA_TRY(cudaStreamSynchronize(s));
     *n_found = total;
     if (total > capacity) {
         set_error("candidate buffer too small: " + std::to_string(total) + " found, capacity " +
@@ -967,10 +980,12 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
     // event interval holds the kernels of one group and nothing else;
     // otherwise the spectrum and correlation run on the plan's
     // high-priority stream (after the work already queued on the caller's)
-    // and the harmonic sums on its low-priority one
-    cudaStream_t hs = p.profiling ? s : p.aux;
+    // and the harmonic sums on its low-priority one.  A single series has
+    // nothing to overlap: everything stays on the caller's stream
+    const bool fork = !p.profiling && n_series > 1;
+    cudaStream_t hs = fork ? p.aux : s;
     cudaStream_t caller = s;
-    if (!p.profiling) {
+    if (fork) {
         FDAS_CUDA_TRY(cudaEventRecord(p.ev_fork, caller));
         FDAS_CUDA_TRY(cudaStreamWaitEvent(p.hi, p.ev_fork, 0));
         s = p.hi;
@@ -1049,10 +1064,7 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
         }
         // plane[b] and partials[b] are free once the harmonic sum of series t-2
         // is done; only the correlation writes them
-        if (t >= 2) {
-            FDAS_CUDA_TRY(cudaStreamWaitEvent(s, p.ev_hsum[b], 0));
-            if (p.profiling) e1 = mark(s);
-        }
+        if (t >= 2 && hs != s) FDAS_CUDA_TRY(cudaStreamWaitEvent(s, p.ev_hsum[b], 0));
         Plan hv = harm_view(v);
         const bool pooled = sums_by_bounds(hv) && v.correlator == FDAS_CORR_TENSOR;
         FDAS_TRY(launch_plane(v, p.spec_pad, p.plane[b], p.partials[b], s,
@@ -1067,15 +1079,17 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
 #endif
         FDAS_DEBUG_CHECK(p, s, "the correlation of series " + std::to_string(t));
         cudaEvent_t e2 = p.profiling ? mark(s) : nullptr;
-        FDAS_CUDA_TRY(cudaEventRecord(p.ev_conv[b], s));
-        FDAS_CUDA_TRY(cudaStreamWaitEvent(hs, p.ev_conv[b], 0));
+        if (hs != s) {
+            FDAS_CUDA_TRY(cudaEventRecord(p.ev_conv[b], s));
+            FDAS_CUDA_TRY(cudaStreamWaitEvent(hs, p.ev_conv[b], 0));
+        }
         cudaEvent_t e3 = p.profiling ? mark(hs) : nullptr;
         TrialStats *ts = p.stats + rank[t];
         FDAS_TRY(launch_finalize_stats(hv, p.partials[b], plane_partials(v), nullptr, ts, hs));
         FDAS_TRY(launch_harmonic_threshold(hv, p.plane[b], b, pooled, ts, (uint32_t)rank[t], hs));
         FDAS_DEBUG_CHECK(p, hs, "the harmonic sum of series " + std::to_string(t));
         cudaEvent_t e4 = p.profiling ? mark(hs) : nullptr;
-        FDAS_CUDA_TRY(cudaEventRecord(p.ev_hsum[b], hs));
+        if (hs != s) FDAS_CUDA_TRY(cudaEventRecord(p.ev_hsum[b], hs));
         p.launches[FDAS_PROF_SPECTRUM] += (v.fft_m1 == 1 ? 1 : 2) + 1;
         p.launches[FDAS_PROF_CORRELATE] += p.interbin ? 2 : 1;   // + fix-up or interbinning
         p.launches[FDAS_PROF_HARMONIC] += 2;
@@ -1089,7 +1103,7 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
         FDAS_CUDA_TRY(cudaEventRecord(p.ev_join, s));
         FDAS_CUDA_TRY(cudaStreamWaitEvent(caller, p.ev_join, 0));
     }
-    for (int b = 0; b < 2 && b < n_series; ++b)
+    for (int b = 0; b < 2 && b < n_series && hs != caller; ++b)
         FDAS_CUDA_TRY(cudaStreamWaitEvent(caller, p.ev_hsum[(n_series - 1 - b) & 1], 0));
     return FDAS_OK;
 }
@@ -1171,12 +1185,7 @@ static fdas_status enqueue_search(Plan &p, const Fault &fault, const fdas_series
         rank[order[i]] = i;
         ids[i] = batch[order[i]].trial_id;
     }
-    // (a copy from pageable memory returns once the source has been read)
-    if (n_series > 0)
-        FDAS_CUDA_TRY(cudaMemcpyAsync(p.rank_ids, ids.data(), sizeof(uint32_t) * n_series,
-                                      cudaMemcpyHostToDevice, s));
-    FDAS_CUDA_TRY(cudaMemsetAsync(p.cand_count, 0, sizeof(unsigned long long), s));
-    FDAS_CUDA_TRY(cudaMemsetAsync(p.flags, 0, sizeof(unsigned int), s));
+    FDAS_TRY(launch_init_search(p, ids.data(), n_series, s));
     if (p.profiling) {
         FDAS_TRY(events_reserve(p, 7 * (size_t)n_series + 2));
         iv.reserve(3 * (size_t)n_series + 1);
@@ -1590,9 +1599,7 @@ fdas_status fdas_threshold(fdas_plan *plan, const void *plane, const double *sta
     const Fault fault = injected_fault();
     if (fault.kind == kFaultUnknown) return fault_args_check(fault);
     p.store_cap = fault.kind == kFaultCapacity ? 1 : p.max_cands;
-    FDAS_CUDA_TRY(cudaMemcpyAsync(p.rank_ids, &trial_id, sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-    FDAS_CUDA_TRY(cudaMemsetAsync(p.cand_count, 0, sizeof(unsigned long long), s));
-    FDAS_CUDA_TRY(cudaMemsetAsync(p.flags, 0, sizeof(unsigned int), s));
+    FDAS_TRY(launch_init_search(p, &trial_id, 1, s));
     Plan hv = harm_view(p);
     FDAS_TRY(launch_finalize_stats(hv, nullptr, 0, stats, p.stats, s));
     FDAS_TRY(launch_harmonic_threshold(hv, plane, 0, false, p.stats, 0, s));
