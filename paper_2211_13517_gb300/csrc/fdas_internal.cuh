@@ -212,7 +212,7 @@ struct Plan {
     uint16_t *pool[2] = {nullptr, nullptr};   // [pool_nb][plane_cols / 2] FP16
     int32_t *pool_blk = nullptr;              // [pool_nb + 1]
     uint32_t *pool_src = nullptr;             // [pool_nb][H]
-    uint2 *pool_masks = nullptr;              // [pool_nb]
+    uint4 *pool_masks = nullptr;              // [pool_nb]
     // boxes that need their exact sums: (bound, block, box) and their number
     unsigned long long *pool_list = nullptr;
     unsigned int pool_list_cap = 0;
@@ -334,7 +334,7 @@ bool sums_by_bounds(const Plan &p);   // whether launch_harmonic_threshold goes 
 constexpr int kPoolMaxRows = 4;   // rows of a block
 std::vector<int32_t> pool_blocks(int n_z);
 bool pool_sources(const std::vector<int32_t> &blk, int n_z, int iz0, int H,
-                  std::vector<uint32_t> *src, std::vector<uint32_t> *masks);
+                  std::vector<uint32_t> *src, std::vector<uint4> *masks);
 fdas_status launch_harmonic_bound(Plan &p, const void *plane, int buf, bool pooled,
                                   const TrialStats *st, uint32_t rank, cudaStream_t s);
 fdas_status launch_harmonic_sums(Plan &p, const void *plane, float *out,

@@ -105,14 +105,17 @@ __global__ void __launch_bounds__(256) pool_kernel(const typename P::real *__res
 }
 
 // ---------------------------------------------------------------------------
-// geometry of the bound sums.  A warp walks consecutive block rows of 1024
-// boxes; lane t owns G = 32 consecutive boxes (64 bins).  Harmonic J of its
+// geometry of the bound sums.  A CTA of W = 8 warps walks down a column of 1024
+// boxes, 8 block rows at a time, one per warp; lane t owns G = 32 consecutive
+// boxes (64 bins) of the warp's row.  Harmonic J of its
 // box i reads the bins from floor((2 i J + H/2)/H) to
 // floor(((2 i + 1) J + H/2)/H) past 64 J t/H, that is one or two consecutive
 // boxes of A at compile-time places past 32 J t/H.  With 32 boxes per lane
 // every window starts on an even box (H <= 16), so pairs of boxes are picked
 // out of whole words with constant selectors.
 // ---------------------------------------------------------------------------
+constexpr int kBoundW = 8;   // warps of a CTA = block rows of a step
+
 template <int H>
 struct Bound {
     static constexpr int G = 32;
@@ -131,7 +134,10 @@ struct Bound {
     static constexpr int words(int J) { return (ne(J) + width(J) - 1) / width(J) * (width(J) / 2); }
     // boxes the warp reads of harmonic J, in whole 16-byte vectors
     static constexpr int len(int J) { return (step(J) * 31 + 2 * words(J) + 7) / 8 * 8; }
-    static constexpr int off(int J) { return J <= 1 ? 0 : off(J - 1) + 2 * len(J - 1); }
+    // source blocks held at a time: those of 8 consecutive block rows (their
+    // rows advance J / H as fast; pool_sources checks the number)
+    static constexpr int slots(int J) { return kBoundW * J / H + 2; }
+    static constexpr int off(int J) { return J <= 1 ? 0 : off(J - 1) + slots(J - 1) * len(J - 1); }
     static constexpr int SMEM_ELEMS = off(H) + 8;   // the top row (J = H) is not staged
 };
 
@@ -209,22 +215,22 @@ struct BoundSteps {
     }
 
     // harmonics j_at(H, IDX), ... in stage order; stage(s, S) after each
-    // stage.  msk.x: bit J - 1 is the slot of harmonic J's (first) source
-    // block, msk.y: its sources span two blocks.
+    // stage.  msk: 4 bits per harmonic (from .x on) with the slot of its (first)
+    // source block, and in .z a bit per harmonic whose sources span two blocks.
     template <int IDX, class F>
     __device__ __forceinline__ static bool sums(const uint16_t *sm, uint64_t *bars, unsigned parity,
-                                                int t, uint2 msk, __half2 (&S)[D::G / 2], F &&stage) {
+                                                int t, uint4 msk, __half2 (&S)[D::G / 2], F &&stage) {
         if constexpr (IDX < H) {
             constexpr int J = j_at(H, IDX);
             if constexpr ((IDX & (IDX - 1)) == 0)
                 if (!mbar_wait(&bars[ilog2h(IDX) + 1], parity)) return false;
             const uint16_t *base = sm + D::off(J);
-            const bool slot1 = (msk.x >> (J - 1)) & 1u;
+            const int slot = (int)(((J <= 8 ? msk.x : msk.y) >> (4 * ((J - 1) & 7))) & 15u);
             uint32_t w[D::words(J)];
-            load_window<J>(base + (slot1 ? D::len(J) : 0), t, w);
-            if ((msk.y >> (J - 1)) & 1u) {
+            load_window<J>(base + slot * D::len(J), t, w);
+            if ((msk.z >> (J - 1)) & 1u) {
                 uint32_t w2[D::words(J)];
-                load_window<J>(base + (slot1 ? 0 : D::len(J)), t, w2);
+                load_window<J>(base + (slot + 1 == D::slots(J) ? 0 : slot + 1) * D::len(J), t, w2);
 #pragma unroll
                 for (int k = 0; k < D::words(J); ++k) w[k] = hmax2_u32(w[k], w2[k]);
             }
@@ -236,45 +242,50 @@ struct BoundSteps {
         }
     }
 
-    // the span lane IDX copies (J = 0: none)
+    // the span lane IDX of warp 0 copies (J = 0: none)
     struct Lane {
-        int J = 0, g = 0, off = 0, len = 0;
+        int J = 0, g = 0, off = 0, len = 0, slots = 1;
     };
     template <int IDX>
     __device__ __forceinline__ static void lane_span(int lane, Lane &L) {
         if constexpr (IDX < H) {
-            constexpr int J = j_at(H, IDX), OFF = D::off(J), LEN = D::len(J);
+            constexpr int J = j_at(H, IDX), OFF = D::off(J), LEN = D::len(J), SLOTS = D::slots(J);
             if (lane == IDX) {
                 L.J = J;
                 L.g = ilog2h(IDX) + 1;
                 L.off = OFF;
                 L.len = LEN;
+                L.slots = SLOTS;
             }
             lane_span<IDX + 1>(lane, L);
         }
     }
 };
 
-// One warp (a CTA of its own) per 1024 boxes of `walk` consecutive block rows.
-// Lane IDX brings harmonic j_at(H, IDX)'s boxes (consecutive: 64 J of a source
-// block at H = 16) to shared memory by a bulk copy when the walk first reaches
-// their source block, into slot (block % 2) of the harmonic, so a source block
-// shared by consecutive rows is copied once.  The copies of a stage complete
-// on the stage's own barrier, one phase per row.
+// Lane IDX of warp 0 brings harmonic j_at(H, IDX)'s boxes (consecutive: 64 J of
+// a source block at H = 16) to shared memory by a bulk copy when the walk first
+// reaches their source block, into slot (block mod slots) of the harmonic, so a
+// source block is copied once per walk.  The copies of a stage complete on the
+// stage's own barrier, one phase per step.  The 8 block rows of a step share the
+// staged blocks: 107 KB for 8 warps at H = 16, two CTAs per SM.
 //
 // A box that reaches a threshold is listed with its last-stage bound (+inf
 // when an earlier stage reached its threshold, which is very rare); `listed`
 // counts them, also beyond the list's capacity.
 //
-// Measured at 2^22 bins x 193 rows, H = 16 (in 49 block rows): 257 us, 7 warps
-// per SM at 1.5 instructions per cycle (31 KB of staged boxes each).  16
-// boxes per lane in CTAs of two warps: 262 us (more instructions per box).
-// Windows exchanged through a small buffer per harmonic from coalesced global
-// loads instead of staged (20 warps per SM): 419 us, bound by the L1.
+// Measured at 2^22 bins x 193 rows, H = 16 (56 block rows): 301 us, 1.6
+// instructions per cycle.  One warp per CTA, with two slots per harmonic of its
+// own (31 KB, 7 warps per SM): 312 us, and half again as slow at H = 8; 16 boxes
+// per lane: a third more instructions, the same time.  A copying warp and 8
+// summing ones that take the next row as soon as the row 8 before it is done
+// (no CTA barrier): 309 us; 2048 boxes per CTA, half the copies: 346 us; the
+// same with 16-byte asynchronous copies instead of bulk ones: 1.2 ms.  Windows
+// exchanged through a small buffer per harmonic from coalesced global loads
+// instead of staged (20 warps per SM): bound by the L1, 419 us.
 template <int H>
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(32 * kBoundW, 2)
     harmonic_bound_kernel(const uint16_t *__restrict__ A, int64_t n_r, int nb, int walk,
-                          const uint32_t *__restrict__ src, const uint2 *__restrict__ masks,
+                          const uint32_t *__restrict__ src, const uint4 *__restrict__ masks,
                           const TrialStats *__restrict__ st, unsigned long long *__restrict__ list,
                           unsigned int list_cap, unsigned int *__restrict__ listed,
                           unsigned int *__restrict__ flags) {
@@ -284,11 +295,11 @@ __global__ void __launch_bounds__(32)
     extern __shared__ __align__(16) unsigned char hb_smem[];
     uint16_t *sm = reinterpret_cast<uint16_t *>(hb_smem);
     __shared__ __align__(8) uint64_t bars[NS + 1];
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t pitch = n_r / 2;
-    const int64_t box0 = (int64_t)blockIdx.x * D::BOXES;   // rows hold whole warps of boxes
+    const int64_t box0 = (int64_t)blockIdx.x * D::BOXES;   // rows hold whole columns of boxes
     const int kb_begin = blockIdx.y * walk, kb_end = min(kb_begin + walk, nb);
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
         for (int g = 0; g <= NS; ++g) mbar_init(&bars[g], 1);
         mbar_fence_init();
     }
@@ -299,15 +310,15 @@ __global__ void __launch_bounds__(32)
         T16[s] = __half2half2(th >= 0.5f && th <= 30000.f ? __float2half_rd(0.99f * th) : __half(0.f));
     }
     typename Steps::Lane sp;
-    Steps::template lane_span<1>(lane, sp);
+    if (warp == 0) Steps::template lane_span<1>(lane, sp);
     const int64_t c0 = sp.J * box0 / H;
     const unsigned bytes = 2u * (unsigned)sp.len;
     int have = -1;   // last source block this lane copied
     bool failed = false;
     int step = 0;
-    // the lane's boxes of the top row and the row's slot bits, one row ahead
+    // the lane's boxes of the top row and the row's slots, one step ahead
     uint4 top[D::G / 8];
-    uint2 msk = make_uint2(0u, 0u);
+    uint4 msk = make_uint4(0u, 0u, 0u, 0u);
     auto load_top = [&](int kb) {
         const int64_t at = kb * pitch + box0 + D::G * lane;
         if (kb < kb_end && FDAS_IN_BOUNDS(at, D::G, nb * pitch, kSiteHsTopLoad)) {
@@ -316,26 +327,35 @@ __global__ void __launch_bounds__(32)
             msk = __ldg(masks + kb);
         }
     };
-    load_top(kb_begin);
+    load_top(kb_begin + warp);
 
-    for (int kb = kb_begin; kb < kb_end; ++kb, ++step) {
-        __syncwarp();   // every lane is done with the last row's boxes
-        if (sp.J != 0) {
-            const uint32_t sb = __ldg(src + kb * H + sp.J - 1);
-            const int sb1 = (int)(sb >> 16);
-            for (int x = max((int)(sb & 0xffffu), have + 1); x <= sb1; ++x) {
-                if (!FDAS_IN_BOUNDS(x, 1, nb, kSiteHsSpanRow) ||
-                    !FDAS_IN_BOUNDS(c0, sp.len, pitch, kSiteHsSpanRange))
-                    continue;
-                fence_proxy_async_smem();
-                mbar_expect_tx(&bars[sp.g], bytes);
-                bulk_copy_g2s(sm + sp.off + (x & 1) * sp.len, A + (int64_t)x * pitch + c0, bytes,
-                              &bars[sp.g]);
-            }
-            have = sb1;
+    for (int kb0 = kb_begin; kb0 < kb_end; kb0 += kBoundW, ++step) {
+        // every warp is done with the last step's boxes (and the barriers are
+        // initialised); stop together after a wait that gave up
+        if (__syncthreads_or(failed)) {
+            failed = true;
+            break;
         }
-        __syncwarp();
-        if (lane >= 1 && lane < NS) mbar_arrive(&bars[lane]);
+        if (warp == 0) {
+            if (sp.J != 0) {
+                const int sb0 = (int)(__ldg(src + kb0 * H + sp.J - 1) & 0xffffu);
+                const int sb1 = (int)(__ldg(src + min(kb0 + kBoundW, kb_end) * H - H + sp.J - 1) >> 16);
+                for (int x = max(sb0, have + 1); x <= sb1; ++x) {
+                    if (!FDAS_IN_BOUNDS(x, 1, nb, kSiteHsSpanRow) ||
+                        !FDAS_IN_BOUNDS(c0, sp.len, pitch, kSiteHsSpanRange))
+                        continue;
+                    fence_proxy_async_smem();
+                    mbar_expect_tx(&bars[sp.g], bytes);
+                    bulk_copy_g2s(sm + sp.off + (x % sp.slots) * sp.len, A + (int64_t)x * pitch + c0,
+                                  bytes, &bars[sp.g]);
+                }
+                have = sb1;
+            }
+            __syncwarp();
+            if (lane >= 1 && lane < NS) mbar_arrive(&bars[lane]);
+        }
+        const int kb = kb0 + warp;
+        if (kb >= kb_end) continue;
         __half2 S[D::G / 2];
 #pragma unroll
         for (int k = 0; k < D::G / 8; ++k) {
@@ -344,8 +364,8 @@ __global__ void __launch_bounds__(32)
             S[4 * k + 2] = as_half2(top[k].z);
             S[4 * k + 3] = as_half2(top[k].w);
         }
-        const uint2 m_now = msk;
-        load_top(kb + 1);
+        const uint4 m_now = msk;
+        load_top(kb + kBoundW);
         uint32_t mask = 0u;    // boxes of this lane that need their exact sums
         uint32_t bound = 0u;   // the largest last-stage bound among them
         auto stage = [&](int s, __half2 (&Sv)[D::G / 2]) {
@@ -366,10 +386,6 @@ __global__ void __launch_bounds__(32)
         stage(0, S);
         if (!Steps::template sums<1>(sm, bars, (unsigned)(step & 1), lane, m_now, S, stage))
             failed = true;
-        if (__any_sync(0xffffffffu, failed)) {
-            failed = true;
-            break;
-        }
         if (__any_sync(0xffffffffu, mask != 0u)) {
             int n = __popc(mask), before = n;
 #pragma unroll
@@ -391,10 +407,12 @@ __global__ void __launch_bounds__(32)
             }
         }
     }
-    if (failed && lane == 0) {
-        atomicOr(flags, 2u);
-        // copies still in flight land before shared memory is released (bounded)
-        for (int g = 1; g < NS; ++g) (void)mbar_wait(&bars[g], (unsigned)(step & 1));
+    if (__syncthreads_or(failed)) {
+        if (threadIdx.x == 0) atomicOr(flags, 2u);
+        // copies still in flight land before shared memory is released (bounded):
+        // those of the last step issued
+        if (threadIdx.x == 0 && step > 0)
+            for (int g = 1; g < NS; ++g) (void)mbar_wait(&bars[g], (unsigned)((step - 1) & 1));
     }
 }
 
@@ -502,13 +520,14 @@ fdas_status launch_bound(Plan &p, const void *plane, int buf, const TrialStats *
     auto k = harmonic_bound_kernel<H>;
     FDAS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const unsigned cols = (unsigned)(p.n_r / 2 / D::BOXES);
-    // block rows per walk: long walks copy each source block once, but the
-    // grid should hold a few warps for every slot of the GPU (7 per SM)
-    const int64_t want = 24 * (int64_t)p.n_sms;
-    const int walks = (int)std::max<int64_t>(1, std::min<int64_t>(p.pool_nb, (want + cols - 1) / cols));
-    const int walk = (p.pool_nb + walks - 1) / walks;
+    // block rows per walk, in whole steps: long walks copy each source block
+    // once, but the grid should fill the GPU (2 CTAs per SM) a few times
+    const int steps = (p.pool_nb + kBoundW - 1) / kBoundW;
+    const int64_t want = 8 * (int64_t)p.n_sms;
+    const int walks = (int)std::max<int64_t>(1, std::min<int64_t>(steps, (want + cols - 1) / cols));
+    const int walk = (steps + walks - 1) / walks * kBoundW;
     dim3 grid(cols, (unsigned)((p.pool_nb + walk - 1) / walk));
-    k<<<grid, 32, smem, s>>>(p.pool[buf], p.n_r, p.pool_nb, walk, p.pool_src, p.pool_masks, st,
+    k<<<grid, 32 * kBoundW, smem, s>>>(p.pool[buf], p.n_r, p.pool_nb, walk, p.pool_src, p.pool_masks, st,
                              p.pool_list, p.pool_list_cap, p.pool_listed, p.flags);
     FDAS_CUDA_TRY(cudaGetLastError());
     const unsigned exact_ctas = std::min(kExactCtas * (unsigned)p.n_sms, p.pool_list_cap / 16);
@@ -548,10 +567,11 @@ std::vector<int32_t> pool_blocks(int n_z) {
 }
 
 // per block and harmonic j = 1..H the first and last source block (16 bits
-// each), and per block the bits (first source block odd, two source blocks);
-// false when the sources of a harmonic span more than two blocks
+// each), and per block the slots of the first ones (4 bits per harmonic) and
+// which harmonics have two; false when the sources do not fit the kernel's
+// slots (two blocks per block row, slots() per step of kBoundW of them)
 bool pool_sources(const std::vector<int32_t> &blk, int n_z, int iz0, int H,
-                  std::vector<uint32_t> *src, std::vector<uint32_t> *masks) {
+                  std::vector<uint32_t> *src, std::vector<uint4> *masks) {
     const int nb = (int)blk.size() - 1;
     std::vector<int32_t> of(n_z);
     for (int i = 0; i < nb; ++i) {
@@ -559,15 +579,19 @@ bool pool_sources(const std::vector<int32_t> &blk, int n_z, int iz0, int H,
         for (int r = blk[i]; r < blk[i + 1]; ++r) of[r] = i;
     }
     src->assign((size_t)nb * H, 0u);
-    masks->assign(2 * (size_t)nb, 0u);
+    masks->assign((size_t)nb, make_uint4(0u, 0u, 0u, 0u));
     for (int i = 0; i < nb; ++i)
         for (int j = 1; j <= H; ++j) {
             const int lo = of[iz0 + src_off(H, blk[i] - iz0, j)];
             const int hi = of[iz0 + src_off(H, blk[i + 1] - 1 - iz0, j)];
             if (hi < lo || hi > lo + 1 || (j == H && (lo != i || hi != i))) return false;
             (*src)[(size_t)i * H + j - 1] = (uint32_t)lo | ((uint32_t)hi << 16);
-            (*masks)[2 * (size_t)i] |= (uint32_t)(lo & 1) << (j - 1);
-            (*masks)[2 * (size_t)i + 1] |= (uint32_t)(hi != lo) << (j - 1);
+            if (j == H) continue;
+            const int slots = kBoundW * j / H + 2, e = std::min(i + kBoundW, nb) - 1;
+            if (of[iz0 + src_off(H, blk[e + 1] - 1 - iz0, j)] - lo + 1 > slots) return false;
+            uint4 &m = (*masks)[i];
+            (j <= 8 ? m.x : m.y) |= (uint32_t)(lo % slots) << (4 * ((j - 1) & 7));
+            m.z |= (uint32_t)(hi != lo) << (j - 1);
         }
     return true;
 }

@@ -513,7 +513,8 @@ static bool bounds_pay(const Plan &p) {
 // the workspace of the sums by bounds for these row blocks (none where they
 // do not pay or a harmonic's sources span more than two blocks)
 static fdas_status build_pool(Plan &p, const std::vector<int32_t> &blk) {
-    std::vector<uint32_t> src, masks;
+    std::vector<uint32_t> src;
+    std::vector<uint4> masks;
     if (!bounds_pay(p) || !pool_sources(blk, p.n_z, p.iz0, p.H, &src, &masks)) return FDAS_OK;
     const int64_t before = p.ws_bytes;
     p.pool_nb = (int)blk.size() - 1;
@@ -525,10 +526,10 @@ static fdas_status build_pool(Plan &p, const std::vector<int32_t> &blk) {
     FDAS_TRY(dalloc(p, &p.pool_listed, sizeof(unsigned int), "pool_listed"));
     FDAS_TRY(dalloc(p, &p.pool_blk, sizeof(int32_t) * blk.size(), "pool_blk"));
     FDAS_TRY(dalloc(p, &p.pool_src, sizeof(uint32_t) * src.size(), "pool_src"));
-    FDAS_TRY(dalloc(p, &p.pool_masks, sizeof(uint32_t) * masks.size(), "pool_masks"));
+    FDAS_TRY(dalloc(p, &p.pool_masks, sizeof(uint4) * masks.size(), "pool_masks"));
     FDAS_CUDA_TRY(cudaMemcpy(p.pool_blk, blk.data(), sizeof(int32_t) * blk.size(), cudaMemcpyHostToDevice));
     FDAS_CUDA_TRY(cudaMemcpy(p.pool_src, src.data(), sizeof(uint32_t) * src.size(), cudaMemcpyHostToDevice));
-    FDAS_CUDA_TRY(cudaMemcpy(p.pool_masks, masks.data(), sizeof(uint32_t) * masks.size(),
+    FDAS_CUDA_TRY(cudaMemcpy(p.pool_masks, masks.data(), sizeof(uint4) * masks.size(),
                              cudaMemcpyHostToDevice));
     p.pool_bytes = p.ws_bytes - before;
     p.pool_on = true;
