@@ -43,7 +43,7 @@ constexpr int kDdThreads = 256;  // 8 warps x 4 DM trials
 constexpr int kDdPer = kDdT / 32;
 constexpr double kDm = 4.148808e3;
 constexpr size_t kDdSmemCap = 200 * 1024;   // both buffers
-constexpr size_t kGrSmem = 220 * 1024;      // by groups: all CTAs of an SM
+constexpr size_t kGrSmem = 222 * 1024;      // by groups: all CTAs of an SM
 
 __global__ void dm_delay_kernel(int32_t *__restrict__ out, int n_chan, int n_dm, double f_top,
                                 double df, double tsamp, double dm_lo, double dm_step) {
@@ -224,9 +224,16 @@ __global__ void __launch_bounds__(kDdThreads, 2)
 // further on, so that odd offsets find aligned words too; 32-bit totals every
 // 64 groups (64 * 4 * 255 < 2^16).  Exact.
 //
-// Bound: instruction issue (about 2.1 per cycle), half of it the pattern sums.
-// Measured: 1024 channels of 8-bit samples, 128 trials, 2^20 outputs 7.35 ms
-// (plain kernel 18.7); 300 FP32 channels, 75 trials, 262181 outputs 0.63 ms
+// Bound: instruction issue (2.4 a cycle) and the two barriers per batch.  With 8-bit
+// samples the pattern sums take 43 % of the time, the trials' additions 26 %,
+// staging and barriers the rest (each part left out in turn).  So a batch takes
+// the groups whose pattern sums fill the 8 warps best (8-bit: 2 pieces of 372
+// samples for 32 trials 71 samples apart, 4 groups; with 3 pieces of 248 samples
+// 6.63 ms below), its sums lie packed in shared memory (a place for the most
+// patterns of any group left room for 2 groups only: 7.04), and what a piece
+// reads again for each pattern stays in registers (7.35 without).
+// Measured: 1024 channels of 8-bit samples, 128 trials, 2^20 outputs 6.07 ms
+// (plain kernel 18.7); 300 FP32 channels, 75 trials, 262181 outputs 0.60 ms
 // (1.32).
 // ---------------------------------------------------------------------------
 constexpr int kGrMax = 4;         // channels per group
@@ -237,50 +244,51 @@ constexpr int kGrFlush = 64;      // groups between 32-bit totals (8-bit samples
 template <class T>
 constexpr int kGrCtas = sizeof(T) == 4 ? 2 : 3;   // CTAs per SM
 template <class T>
-constexpr int kGrChunk = sizeof(T) == 4 ? 160 : 248;
+constexpr int kGrChunk = sizeof(T) == 4 ? 160 : 372;
 constexpr int kGrPer = 5;         // FP32 samples of a chunk per lane
 
 // one group of a DM tile as the kernel reads it (whole 16-byte copies)
 struct GrRec {
-    int32_t c0, nk, np, pad;      // first channel, channels, patterns
-    int16_t pat[kGrPat][4];       // [0]: first channel that differs from the pattern
-                                  // before; [k]: shift of channel k
-    // per DM the first word of its samples among the group's pattern sums, of
+    int32_t c0, nk;               // first channel, channels
+    int16_t np, y0[2], pad;       // patterns; patterns of the batch's groups before (FP32, 8-bit)
+    int32_t first[kGrMax];        // delay of channel k in the tile's first trial
+    int16_t pat[kGrPat + 2][4];   // [0]: first channel that differs from the pattern
+                                  // before; [k]: shift of channel k (one is read ahead)
+    // per DM the first word of its samples among the batch's pattern sums, of
     // FP32 and of 8-bit samples (words of two; odd offsets in the second copy)
     int32_t off[2][kDdD];
 };
 static_assert(sizeof(GrRec) % 16 == 0, "whole 16-byte copies");
 
-// 8 samples (four 16-bit pairs) of an 8-bit window from byte `at` + 8 lane on
-__device__ __forceinline__ void add8_u8(const uint8_t *x, int at, int lane, uint32_t (&v)[4]) {
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(x) + (at >> 2) + 2 * lane;
-    const uint32_t a = w[0], b = w[1], c = w[2];
+// 12 samples (six 16-bit pairs) of an 8-bit window from byte `at` + 12 lane on
+__device__ __forceinline__ void add12_u8(const uint8_t *x, int at, int lane, uint32_t (&v)[6]) {
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(x) + (at >> 2) + 3 * lane;
+    const uint32_t a[4] = {w[0], w[1], w[2], w[3]};
     const unsigned sh = 8u * (unsigned)(at & 3);
-    const uint32_t lo = __funnelshift_r(a, b, sh), hi = __funnelshift_r(b, c, sh);
-    v[0] += __byte_perm(lo, 0u, 0x4140u);
-    v[1] += __byte_perm(lo, 0u, 0x4342u);
-    v[2] += __byte_perm(hi, 0u, 0x4140u);
-    v[3] += __byte_perm(hi, 0u, 0x4342u);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const uint32_t b = __funnelshift_r(a[i], a[i + 1], sh);
+        v[2 * i] += __byte_perm(b, 0u, 0x4140u);
+        v[2 * i + 1] += __byte_perm(b, 0u, 0x4342u);
+    }
 }
 
 // shared-memory geometry: per slot the channel windows (xpitch bytes each) and
 // the batch's records; then the pattern sums (ypitch words each)
 template <class T>
 __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
-    dedisperse_group_kernel(const T *__restrict__ fb, const int32_t *__restrict__ delays,
-                            const GrRec *__restrict__ recs, const int32_t *__restrict__ n_groups,
-                            int max_groups, float *__restrict__ out, int n_chan, int64_t n_t,
-                            int n_dm, int64_t n_out, int chunks, int lead, int xpitch, int ypitch,
-                            int max_pat, int batch) {
+    dedisperse_group_kernel(const T *__restrict__ fb, const GrRec *__restrict__ recs,
+                            const int32_t *__restrict__ n_groups, int max_groups,
+                            float *__restrict__ out, int64_t n_t, int n_dm, int64_t n_out, int chunks,
+                            int lead, int xpitch, int ypitch, int batch) {
     constexpr bool kU8 = sizeof(T) == 1;
     extern __shared__ __align__(16) unsigned char dd_smem[];
     const int slot_bytes = batch * (kGrMax * xpitch + (int)sizeof(GrRec));
     uint32_t *const Y = reinterpret_cast<uint32_t *>(dd_smem + 2 * slot_bytes);
-    __shared__ int32_t shift[2][kGrBatchMax * kGrMax];   // of each window's first sample
+    __shared__ __align__(16) int32_t shift[2][kGrBatchMax * kGrMax];   // of each window's first sample
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t t0 = (int64_t)blockIdx.x * kDdT;
     const int d_lo = blockIdx.y * kDdD;
-    const int32_t *dl = delays + (int64_t)d_lo * n_chan;
     const GrRec *rec = recs + (int64_t)blockIdx.y * max_groups;
     const int ng = n_groups[blockIdx.y];
     auto slot_rec = [&](int slot) {
@@ -296,11 +304,13 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
         // one warp per channel
         for (int i = warp; i < n * kGrMax; i += kDdThreads / 32) {
             const int g = i / kGrMax, k = i % kGrMax;
-            if (k >= __ldg(&rec[g0 + g].nk)) continue;
-            const int c = __ldg(&rec[g0 + g].c0) + k;
+            const int2 head = __ldg(reinterpret_cast<const int2 *>(rec + g0 + g));   // c0, nk
+            const int delay = __ldg(&rec[g0 + g].first[k]);
+            if (k >= head.y) continue;
+            const int c = head.x + k;
             // the window starts `lead` samples early (shifts may be negative),
             // rounded down to an address of a multiple of 16 bytes
-            const int64_t first = t0 + __ldg(dl + c) - lead;
+            const int64_t first = t0 + delay - lead;
             const T *src = fb + (int64_t)c * n_t;
             constexpr int kV = 16 / (int)sizeof(T);
             const int a = (int)((reinterpret_cast<uintptr_t>(src + first) / sizeof(T)) % kV);
@@ -363,6 +373,9 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
         }
     };
 
+    // the warp's first piece of pattern sums and the step to its next one
+    const int g_first = warp / chunks, ch_first = warp - g_first * chunks;
+    const int g_step = (kDdThreads / 32) / chunks, ch_step = kDdThreads / 32 - g_step * chunks;
     stage(0, 0);
     int slot = 0;
     for (int g0 = 0; g0 < ng; g0 += batch, slot ^= 1) {
@@ -372,25 +385,30 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
         if (g0 + batch < ng) stage(g0 + batch, slot ^ 1);
         const GrRec *r = slot_rec(slot);
         // pattern sums: one warp per group and kGrChunk samples
-        for (int it = warp; it < n * chunks; it += kDdThreads / 32) {
-            const int g = it / chunks, ch = it - g * chunks;
+        for (int g = g_first, ch = ch_first; g < n;) {
             const int np = r[g].np, nk = r[g].nk;
             const unsigned char *xs = dd_smem + slot * slot_bytes + g * kGrMax * xpitch;
-            const int32_t *sh = shift[slot] + g * kGrMax;
+            // where each channel's samples start (kept in registers: the stores
+            // of the sums would have them read again for every pattern)
+            const int4 sh = *reinterpret_cast<const int4 *>(shift[slot] + g * kGrMax);
+            short4 next = *reinterpret_cast<const short4 *>(r[g].pat[0]);
             if constexpr (!kU8) {
                 // lane: samples chunk start + lane + 32 j
-                const float *xw = reinterpret_cast<const float *>(xs) + kGrChunk<T> * ch + lane;
-                float *y = reinterpret_cast<float *>(Y) + g * max_pat * ypitch + kGrChunk<T> * ch + lane;
+                const int at_y = kGrChunk<T> * ch + lane;   // (past ypitch nothing is read)
+                const float *xw = reinterpret_cast<const float *>(xs) + at_y;
+                float *y = reinterpret_cast<float *>(Y) + r[g].y0[0] * ypitch + at_y;
                 float p0[kGrPer], p1[kGrPer], p2[kGrPer];
                 {
-                    const float *w = xw + sh[0];
+                    const float *w = xw + sh.x;
 #pragma unroll
                     for (int j = 0; j < kGrPer; ++j) p0[j] = w[32 * j];
                 }
                 // v = u + channel k at shift s (u itself past the group's channels)
+                const int at[kGrMax] = {0, xpitch / 4 + sh.y, 2 * (xpitch / 4) + sh.z,
+                                        3 * (xpitch / 4) + sh.w};
                 auto x = [&](int k, int s, const float (&u)[kGrPer], float (&v)[kGrPer]) {
                     if (k < nk) {
-                        const float *w = xw + k * (xpitch / 4) + sh[k] + s;
+                        const float *w = xw + at[k] + s;
 #pragma unroll
                         for (int j = 0; j < kGrPer; ++j) v[j] = u[j] + w[32 * j];
                     } else {
@@ -399,40 +417,60 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
                     }
                 };
                 for (int p = 0; p < np; ++p, y += ypitch) {
-                    const short4 pt = *reinterpret_cast<const short4 *>(r[g].pat[p]);
+                    const short4 pt = next;
+                    next = *reinterpret_cast<const short4 *>(r[g].pat[p + 1]);
                     if (pt.x <= 1) x(1, pt.y, p0, p1);
                     if (pt.x <= 2) x(2, pt.z, p1, p2);
                     float v[kGrPer];
                     x(3, pt.w, p2, v);
 #pragma unroll
-                    for (int j = 0; j < kGrPer; ++j) y[32 * j] = v[j];
+                    for (int j = 0; j < kGrPer; ++j)
+                        if (at_y + 32 * j < ypitch) y[32 * j] = v[j];
                 }
             } else {
-                // lane: samples 248 ch + 8 lane .. + 7 as four pairs; lane 31 only
-                // hands its first sample to lane 30
-                uint32_t *y = Y + g * max_pat * 2 * ypitch + 124 * ch + 4 * lane;
-                uint32_t p0[4] = {0u, 0u, 0u, 0u}, p1[4], p2[4];
-                add8_u8(xs, sh[0] + 248 * ch, lane, p0);
-                auto x = [&](int k, int s, const uint32_t (&u)[4], uint32_t (&v)[4]) {
+                // lane: samples 372 ch + 12 lane .. + 11 as six pairs (an odd number
+                // of words per lane: no bank conflicts); lane 31 only hands its
+                // first sample to lane 30
+                constexpr int kC = kGrChunk<T>;
+                const bool store = lane < 31 && kC / 2 * ch + 6 * lane < ypitch;
+                uint32_t *y = Y + r[g].y0[1] * 2 * ypitch + kC / 2 * ch + 6 * lane;
+                uint32_t p0[6] = {0u, 0u, 0u, 0u, 0u, 0u}, p1[6], p2[6];
+                // (windows start on multiples of 16 bytes, so a window's place can
+                // go into the byte offset)
+                const int at[kGrMax] = {sh.x + kC * ch, xpitch + sh.y + kC * ch,
+                                        2 * xpitch + sh.z + kC * ch, 3 * xpitch + sh.w + kC * ch};
+                add12_u8(xs, at[0], lane, p0);
+                auto x = [&](int k, int s, const uint32_t (&u)[6], uint32_t (&v)[6]) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) v[j] = u[j];
-                    if (k < nk) add8_u8(xs + k * xpitch, sh[k] + s + 248 * ch, lane, v);
+                    for (int j = 0; j < 6; ++j) v[j] = u[j];
+                    if (k < nk) add12_u8(xs, at[k] + s, lane, v);
                 };
                 for (int p = 0; p < np; ++p, y += 2 * ypitch) {
-                    const short4 pt = *reinterpret_cast<const short4 *>(r[g].pat[p]);
+                    const short4 pt = next;
+                    next = *reinterpret_cast<const short4 *>(r[g].pat[p + 1]);
                     if (pt.x <= 1) x(1, pt.y, p0, p1);
                     if (pt.x <= 2) x(2, pt.z, p1, p2);
-                    uint32_t v[4];
+                    uint32_t v[6];
                     x(3, pt.w, p2, v);
                     const uint32_t nx = __shfl_down_sync(0xffffffffu, v[0], 1);
-                    if (lane < 31) {
-                        *reinterpret_cast<uint4 *>(y) = make_uint4(v[0], v[1], v[2], v[3]);
-                        // and one sample further on
-                        *reinterpret_cast<uint4 *>(y + ypitch) = make_uint4(
-                            __byte_perm(v[0], v[1], 0x5432u), __byte_perm(v[1], v[2], 0x5432u),
-                            __byte_perm(v[2], v[3], 0x5432u), __byte_perm(v[3], nx, 0x5432u));
+                    if (store) {
+#pragma unroll
+                        for (int j = 0; j < 6; j += 2) {
+                            const uint32_t after = j == 4 ? nx : v[j + 2];
+                            *reinterpret_cast<uint2 *>(y + j) = make_uint2(v[j], v[j + 1]);
+                            // and one sample further on
+                            *reinterpret_cast<uint2 *>(y + ypitch + j) =
+                                make_uint2(__byte_perm(v[j], v[j + 1], 0x5432u),
+                                           __byte_perm(v[j + 1], after, 0x5432u));
+                        }
                     }
                 }
+            }
+            ch += ch_step;
+            g += g_step;
+            if (ch >= chunks) {
+                ch -= chunks;
+                ++g;
             }
         }
         __syncthreads();
@@ -440,14 +478,13 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
         if constexpr (!kU8) {
             for (int g = 0; g < n; ++g) {
                 const int4 o = *reinterpret_cast<const int4 *>(r[g].off[0] + 4 * warp);
-                const float *y = reinterpret_cast<const float *>(Y) + g * max_pat * ypitch + lane;
+                const float *y = reinterpret_cast<const float *>(Y) + lane;
                 add_pair(y, o.x, o.y, acc[0], acc[1]);
                 add_pair(y, o.z, o.w, acc[2], acc[3]);
             }
         } else {
             // two groups per addition
             const uint32_t *y = Y + lane;
-            const int per = 2 * max_pat * ypitch;
             int g = 0;
             for (; g + 1 < n; g += 2) {
                 const int4 oa = *reinterpret_cast<const int4 *>(r[g].off[1] + 4 * warp);
@@ -455,7 +492,7 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
                 const int wa[4] = {oa.x, oa.y, oa.z, oa.w}, wb[4] = {ob.x, ob.y, ob.z, ob.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const uint32_t *a = y + g * per + wa[q], *b = y + (g + 1) * per + wb[q];
+                    const uint32_t *a = y + wa[q], *b = y + wb[q];
 #pragma unroll
                     for (int k = 0; k < kDdPer / 2; ++k) part[q][k] += a[32 * k] + b[32 * k];
                 }
@@ -465,7 +502,7 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
                 const int wa[4] = {oa.x, oa.y, oa.z, oa.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const uint32_t *a = y + g * per + wa[q];
+                    const uint32_t *a = y + wa[q];
 #pragma unroll
                     for (int k = 0; k < kDdPer / 2; ++k) part[q][k] += a[32 * k];
                 }
@@ -526,8 +563,9 @@ void group_tile(const int32_t *delays, int n_chan, int d0, int d1, int chunks, s
             GrRec r{};
             r.c0 = c;
             r.nk = nk;
-            r.np = (int)pats.size();
+            r.np = (int16_t)pats.size();
             int nodes = 1;
+            for (int k = 0; k < nk; ++k) r.first[k] = base[k];
             for (int p = 0; p < r.np; ++p) {
                 int first = 1;
                 if (p > 0)
@@ -572,34 +610,51 @@ struct DedispPlan {
     bool grouped = false;
     GrRec *recs = nullptr;          // device [tiles][max_groups]
     int32_t *n_groups = nullptr;    // device [tiles]
-    int32_t max_groups = 0, max_pat = 1, lead = 0, tail = 0;
+    int32_t max_groups = 0, lead = 0, tail = 0;
+    int32_t batch[2] = {0, 0}, batch_pat[2] = {0, 0};   // FP32, 8-bit: groups and most patterns of a batch
     int64_t table_bytes = 0;
 };
 
-// bytes of a channel window, words of a pattern sum and groups per batch
+// pieces of a pattern sum, bytes of a channel window, words of a pattern sum,
+// and the shared memory of `batch` groups with `pats` patterns
 template <class T>
-static void group_layout(const DedispPlan &p, int *chunks, int *xpitch, int *ypitch, int *batch,
-                         size_t *smem) {
-    *chunks = (kDdT + p.span + kGrChunk<T> - 1) / kGrChunk<T>;
-    // samples a window is read over, from up to 15 bytes past a 16-byte boundary
-    // (8-bit: lane 31's samples and a word past them too)
-    const int len = kGrChunk<T> * *chunks + p.lead + p.tail + (sizeof(T) == 4 ? 3 : 15 + 16);
-    *xpitch = ((int)sizeof(T) * len + 15) / 16 * 16;
-    *ypitch = sizeof(T) == 4 ? kGrChunk<T> * *chunks : (kGrChunk<T> / 2) * *chunks;
-    const size_t per = 2 * (kGrMax * (size_t)*xpitch + sizeof(GrRec)) +
-                       4 * (size_t)p.max_pat * *ypitch * (sizeof(T) == 4 ? 1 : 2);
-    // as many groups as fill the warps of the pattern sums best
-    const int warps = kDdThreads / 32, most = (int)std::min<size_t>(kGrBatchMax, kGrSmem / kGrCtas<T> / per);
-    *batch = 0;
+static size_t group_layout(const DedispPlan &p, int batch, int pats, int *chunks, int *xpitch,
+                           int *ypitch) {
+    const int len = kDdT + p.span;   // samples that the DM trials read
+    *chunks = (len + kGrChunk<T> - 1) / kGrChunk<T>;
+    // (from up to 15 bytes past a 16-byte boundary.  Lanes past `len` read on into
+    // what follows, at most a chunk, and store nothing: the records and sums
+    // behind the last window are longer)
+    *xpitch = ((int)sizeof(T) * (len + p.lead + p.tail) + 15 + 15) / 16 * 16;
+    *ypitch = sizeof(T) == 4 ? len : (len + 11) / 12 * 6;   // (whole lanes)
+    return 2 * (size_t)batch * (kGrMax * (size_t)*xpitch + sizeof(GrRec)) +
+           4 * (size_t)pats * *ypitch * (sizeof(T) == 4 ? 1 : 2);
+}
+
+// groups per batch: as many as fill the warps of the pattern sums best, in the
+// shared memory of the fullest batch
+template <class T>
+static void choose_batch(DedispPlan &p, const std::vector<std::vector<GrRec>> &tiles) {
+    constexpr int kIdx = sizeof(T) == 4 ? 0 : 1;
+    const int warps = kDdThreads / 32;
     double best = 0.0;
-    for (int b = 1; b <= most; ++b) {
-        const double fill = (double)b * *chunks / (warps * ((b * *chunks + warps - 1) / warps));
+    for (int b = 1; b <= kGrBatchMax; ++b) {
+        int pats = 0;
+        for (const std::vector<GrRec> &recs : tiles)
+            for (size_t g = 0; g < recs.size(); g += b) {
+                int n = 0;
+                for (size_t i = g; i < std::min(recs.size(), g + b); ++i) n += recs[i].np;
+                pats = std::max(pats, n);
+            }
+        int chunks, xp, yp;
+        if (group_layout<T>(p, b, pats, &chunks, &xp, &yp) > kGrSmem / kGrCtas<T>) break;
+        const double fill = (double)b * chunks / (warps * ((b * chunks + warps - 1) / warps));
         if (fill >= best) {
             best = fill;
-            *batch = b;
+            p.batch[kIdx] = b;
+            p.batch_pat[kIdx] = pats;
         }
     }
-    *smem = per * (size_t)*batch;
 }
 
 template <class T>
@@ -610,15 +665,16 @@ fdas_status launch_dedisperse(DedispPlan &p, const T *filterbank, float *out, cu
     dim3 grid((unsigned)((p.n_out + kDdT - 1) / kDdT), (unsigned)((p.n_dm + kDdD - 1) / kDdD));
     cudaError_t e;
     if (p.grouped) {
-        int chunks, xpitch, ypitch, batch;
-        size_t smem;
-        group_layout<T>(p, &chunks, &xpitch, &ypitch, &batch, &smem);
+        constexpr int kIdx = sizeof(T) == 4 ? 0 : 1;
+        const int batch = p.batch[kIdx];
+        int chunks, xpitch, ypitch;
+        const size_t smem = group_layout<T>(p, batch, p.batch_pat[kIdx], &chunks, &xpitch, &ypitch);
         e = cudaFuncSetAttribute(dedisperse_group_kernel<T>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess) {
             dedisperse_group_kernel<T><<<grid, kDdThreads, smem, s>>>(
-                filterbank, p.delays, p.recs, p.n_groups, p.max_groups, out, p.n_chan, p.n_t, p.n_dm,
-                p.n_out, chunks, p.lead, xpitch, ypitch, p.max_pat, batch);
+                filterbank, p.recs, p.n_groups, p.max_groups, out, p.n_t, p.n_dm,
+                p.n_out, chunks, p.lead, xpitch, ypitch, batch);
             e = cudaGetLastError();
         }
         if (cur != p.device) cudaSetDevice(cur);
@@ -748,27 +804,36 @@ fdas_status fdas_dedisp_plan_create(fdas_dedisp_plan **out, int32_t n_chan, int6
                 plain += 16.0 * (d1 - d0) * n_chan;
                 counts[t] = (int32_t)per[t].size();
                 most = std::max(most, per[t].size());
-                for (const fdas::GrRec &r : per[t]) p->max_pat = std::max(p->max_pat, r.np);
             }
             p->lead = -shape.lo;
             p->tail = shape.hi;
-            int nc, xp, ypf, ypu, bf, bu;
-            size_t sm;
-            fdas::group_layout<float>(*p, &nc, &xp, &ypf, &bf, &sm);
-            fdas::group_layout<uint8_t>(*p, &nc, &xp, &ypu, &bu, &sm);
+            fdas::choose_batch<float>(*p, per);
+            fdas::choose_batch<uint8_t>(*p, per);
+            const int bf = p->batch[0], bu = p->batch[1];
+            int nc, xp, ypf, ypu;
+            fdas::group_layout<float>(*p, bf, p->batch_pat[0], &nc, &xp, &ypf);
+            fdas::group_layout<uint8_t>(*p, bu, p->batch_pat[1], &nc, &xp, &ypu);
             // (accesses of the pattern sums and of the trials against the plain
             // kernel's one per addition; at equal counts the extra barriers and
             // table reads make groups slower)
             if (shape.cost < 0.75 * plain && bf >= 1 && bu >= 1 && span < (1 << 24)) {
                 std::vector<fdas::GrRec> flat(most * (size_t)tiles);
-                for (int t = 0; t < tiles; ++t)
-                    std::copy(per[t].begin(), per[t].end(), flat.begin() + (size_t)t * most);
-                for (fdas::GrRec &r : flat)
-                    for (int d = 0; d < fdas::kDdD; ++d) {
-                        const int pat = r.off[0][d], off = r.off[1][d];
-                        r.off[0][d] = pat * ypf + off;
-                        r.off[1][d] = (2 * pat + (off & 1)) * ypu + off / 2;
+                for (int t = 0; t < tiles; ++t) {
+                    int y0[2] = {0, 0};   // patterns of the batch so far
+                    for (size_t g = 0; g < per[t].size(); ++g) {
+                        fdas::GrRec &r = flat[(size_t)t * most + g] = per[t][g];
+                        for (int i = 0; i < 2; ++i) {
+                            if (g % (size_t)p->batch[i] == 0) y0[i] = 0;
+                            r.y0[i] = (int16_t)y0[i];
+                        }
+                        for (int d = 0; d < fdas::kDdD; ++d) {
+                            const int pat = r.off[0][d], off = r.off[1][d];
+                            r.off[0][d] = (y0[0] + pat) * ypf + off;
+                            r.off[1][d] = (2 * (y0[1] + pat) + (off & 1)) * ypu + off / 2;
+                        }
+                        for (int &y : y0) y += r.np;
                     }
+                }
                 p->table_bytes = (int64_t)(sizeof(fdas::GrRec) * flat.size() + sizeof(int32_t) * tiles);
                 e = cudaMalloc(&p->recs, sizeof(fdas::GrRec) * flat.size());
                 if (e == cudaSuccess) e = cudaMalloc(&p->n_groups, sizeof(int32_t) * tiles);
