@@ -163,6 +163,7 @@ def work_model(info, prec_bytes):
     n, n_r, n_z, L, H = info.n_samples, info.n_r, info.n_z, info.seg_len, info.n_harm
     gather = sum((j / H) ** 2 for j in range(1, H + 1))
     plane = b_p * n_z * n_r
+    pool = 2 * math.ceil(n_z / 4) * (n_r // 2)   # FP16 maxima of 2 bins x 4 rows
     return {
         # series read + spectrum write (FFT intermediates stay in L2)
         "spectrum_bytes": 4 * n + b_s * n_r,
@@ -176,12 +177,13 @@ def work_model(info, prec_bytes):
             for i in range(n_z)),
         # harmonic gathers: unique cells of stream j are (j/H)^2 of the plane
         "harmonic_bytes": plane * gather,
-        # what the harmonic sum must read from memory at least: the plane once
-        "harmonic_min_bytes": plane,
+        # what the sums by bounds must read from memory at least: the pooled
+        # plane once (the plane itself only where a bound reaches a threshold)
+        "harmonic_min_bytes": pool,
         "alg_bytes": 4 * n + 2 * b_s * n_r + plane * (1 + gather),
         # floor of the whole path: series read, spectrum written and read,
-        # plane written once and read once
-        "min_bytes": 4 * n + 2 * b_s * n_r + 2 * plane,
+        # plane written once, pooled plane written and read
+        "min_bytes": 4 * n + 2 * b_s * n_r + plane + 2 * pool,
     }
 
 
@@ -587,19 +589,20 @@ def run_gpu(args, rank, world, local_rank, dist):
         if group == "harmonic":
             t_hs = k_bf16["harmonic"]["ms_per_trial"] / 1e3
             ach = wm["harmonic_min_bytes"] / t_hs / 1e9
-            return {"kernel": "harmonic_dedup_kernel<BF16,16>", "bound": "hbm",
+            return {"kernel": "harmonic_bound_kernel<16>", "bound": "hbm",
                     "achieved": ach, "peak": peak_hbm, "unit": "GB/s",
                     "frac": ach / peak_hbm, "traffic": traffic,
                     "peak_source": f"{peak_src} hbm_gbs (MEASURED_PEAKS.json)",
-                    "work": "the plane read once (1.62 GB BF16 per trial), the least the "
-                            "harmonic sum must read from HBM",
+                    "work": "the pooled plane read once (0.21 GB per trial), the least the "
+                            "harmonic sum by bounds must read from HBM",
                     "gathers": {"bytes_per_trial": wm["harmonic_bytes"],
                                 "achieved_gbs": k_bf16["harmonic"]["gbs"],
                                 "l2_copy_gbs": l2_gbs,
                                 "frac_of_l2_copy": k_bf16["harmonic"]["gbs"] / l2_gbs,
-                                "note": "plane x sum_j (j/H)^2 = 5.84 planes of gathered BF16 "
-                                        "cells, most served from L2; l2_copy_gbs is a torch copy "
-                                        "of an L2-resident 32 MiB buffer (read + write bytes)"}}
+                                "note": "plane x sum_j (j/H)^2 = 5.84 planes of BF16 cells that "
+                                        "the plain sum would gather and the bounds rule out; "
+                                        "l2_copy_gbs is a torch copy of an L2-resident 32 MiB "
+                                        "buffer (read + write bytes)"}}
         a = k_bf16["correlate"]["tflops"]
         if tensor:
             return {"kernel": "correlate_tc_kernel<BF16> (tcgen05)", "bound": "tensor",
@@ -645,12 +648,13 @@ def run_gpu(args, rank, world, local_rank, dist):
         "roofline_other": other,
         "hbm_alg": {"bytes_per_trial": wm["alg_bytes"], "achieved_gbs": alg_gbs,
                     "peak_gbs": peak_hbm, "frac": alg_gbs / peak_hbm,
-                    "note": f"B_alg (5.84 plane-equivalents of harmonic gathers, mostly L2 "
-                            f"hits) of the whole path / step time, {peak_src} peak"},
+                    "note": f"B_alg (with the 5.84 plane-equivalents of harmonic gathers of the "
+                            f"plain sum, which the bounds mostly rule out) of the whole path / "
+                            f"step time, {peak_src} peak"},
         "hbm_min": {"bytes_per_trial": wm["min_bytes"], "achieved_gbs": min_gbs,
                     "frac": min_gbs / peak_hbm,
-                    "note": "B_min: series read, spectrum written + read, plane written once "
-                            "and read once, over the step time"},
+                    "note": "B_min: series read, spectrum written + read, plane written once, "
+                            "pooled plane written and read, over the step time"},
         "hbm_ncu": ({"bytes_per_trial": ncu_bytes, "achieved_gbs": ncu_bytes / t_trial / 1e9,
                      "frac": ncu_bytes / t_trial / 1e9 / peak_hbm,
                      "note": "DRAM read + write bytes of the correlation and harmonic kernels "
@@ -811,9 +815,9 @@ def run_dedisp(args, dev, capi, world):
            "roofline": {"bound": "smem", "achieved": adds / (ms / 1000.0) / 1e12,
                         "peak": SMEM_WORDS_PEAK_T, "unit": "T additions/s",
                         "frac": adds / (ms / 1000.0) / 1e12 / SMEM_WORDS_PEAK_T},
-           "note": "dedisperse_kernel, inputs larger than L2 (filterbank 34 GB); one 4-byte "
-                   "shared-memory word per addition is the bound (less where two DM trials "
-                   "share a delay)"}
+           "note": "dedisperse_group_kernel, inputs larger than L2 (filterbank 34 GB); peak is "
+                   "one 4-byte shared-memory word per addition; sums shared by the trials of a "
+                   "channel group need fewer"}
     # the same trials from an 8-bit filterbank (the usual format; exact sums),
     # then the whole chain: 8-bit filterbank -> DM-trial series -> BF16 search
     del fb

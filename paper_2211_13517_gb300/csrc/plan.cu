@@ -497,13 +497,14 @@ static Plan plan_view(const Plan &p, int64_t n) {
 
 // Whether the harmonic sum goes by bounds (harmonic_bound.cu).  It adds the
 // pooled plane and two kernels, and pays when few bounds reach a threshold and
-// the plane is more than a few rows: a BF16 search of 2^22 samples x 193 rows,
-// 16 harmonics, against the plain kernel: 6 sigma 738 us (1029), 5.5 sigma 866
-// (1038), 5 sigma 1138 (1072); 8 harmonics: 6 sigma 586 (771), 5 sigma 648
-// (800), 4.5 sigma 1004 (998).  One harmonic only compares cells (308 against
-// 288), and with one row the extra launches cost 10 to 15 us.  Unnormalised
-// planes and the mean + k sigma rule (far lower thresholds) keep the plain
-// kernel.
+// the plane is more than a few rows.  A BF16 search of 2^22 samples x 193 rows
+// (whole call, us; by the plain kernel in brackets, measured with the rule
+// switched): 16 harmonics, 6 sigma 504 (1029), 5.5 sigma 591 (1038), 5 sigma
+// longer by bounds than plain (1138 against 1072 when the rule was set); 8
+// harmonics, 6 sigma 417 (771), 5 sigma 440 (800), 4.5 sigma even then (1004,
+// 998).  One harmonic only compares cells (308 against 288), and with one row
+// the extra launches cost 10 to 15 us.  Unnormalised planes and the mean + k
+// sigma rule (far lower thresholds) keep the plain kernel.
 static bool bounds_pay(const Plan &p) {
     return p.harm_mode == FDAS_HARM_TOP && p.H >= 2 && p.H <= 16 && p.n_z >= 12 &&
            p.norm_mode == FDAS_NORM_MEDIAN && p.thr_mode == FDAS_THRESH_GAMMA_TAIL &&
