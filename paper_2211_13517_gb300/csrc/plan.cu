@@ -947,10 +947,12 @@ static bool is_pinned_or_device(const void *ptr) {
 // to stall intermittently (a search of 64 series from 100 to 135-145 ms)
 // once other processes had churned the host's memory, while these loads
 // kept their rate (100.5 ms, against 99.6 ms for device-resident series);
-// pageable memory still goes through cudaMemcpyAsync.  Eight CTAs keep the
-// copy ahead of the kernels while taking the fewest SM slots from them (32
-// and 152 CTAs measured 101.5 and 106.8 ms).
-constexpr int kH2dCtas = 8, kH2dThreads = 512;
+// pageable memory still goes through cudaMemcpyAsync.  24 CTAs: a BF16 search of
+// page-locked series of 2^23 samples x 193 rows takes 0.851 ms a series (0.794
+// device-resident; 16 CTAs 0.853, 40 0.853, 8 0.852 to 0.886 from box to box,
+// their copy being about as slow as the kernels it runs beside; 64 or 128 CTAs
+// of a quarter of the threads 0.857 and 0.854).
+constexpr int kH2dCtas = 24, kH2dThreads = 512;
 __global__ void __launch_bounds__(kH2dThreads) h2d_copy_kernel(float4 *__restrict__ dst,
                                                                const float4 *__restrict__ src,
                                                                int64_t n4) {
