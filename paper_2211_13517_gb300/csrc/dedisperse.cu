@@ -324,10 +324,13 @@ __global__ void __launch_bounds__(kDdThreads, kGrCtas<T>)
             }
             for (int j = lane; j < xpitch / 16; j += 32) {
                 const int64_t s = first - a + kV * j;
-                if (s >= 0) {
+                if (s >= n_t) {
+                    // past the last sample: no copy, whose address would have to be
+                    // inside the row and aligned (rows start anywhere on 4 bytes)
+                    *reinterpret_cast<uint4 *>(dst + kV * j) = make_uint4(0u, 0u, 0u, 0u);
+                } else if (s >= 0) {
                     const int64_t left = n_t - s;
-                    const int valid = left <= 0 ? 0 : (left >= kV ? 16 : (int)left * (int)sizeof(T));
-                    cp_async16(dst + kV * j, src + (valid > 0 ? s : 0), valid);
+                    cp_async16(dst + kV * j, src + s, left >= kV ? 16 : (int)left * (int)sizeof(T));
                 } else {
                     // before the first sample: zeros, then element by element
 #pragma unroll

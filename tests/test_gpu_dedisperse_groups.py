@@ -54,3 +54,25 @@ def test_grouped_sums(capi, bits, n_chan, n_t, n_out, df, dm_lo, dm_step, n_dm):
         bound = O.dedisperse(np.abs(fb.astype(np.float64)), delays, n_out) * (n_chan - 1) * 2.0 ** -24
         assert np.all(np.abs(got - ref) <= bound + 1e-6)
     plan.close()
+
+
+@pytest.mark.parametrize("off", [0, 1, 3])   # the filterbank's first sample, in elements past 16 bytes
+@pytest.mark.parametrize("n_t", [2048, 2049, 2050, 2051])
+def test_rows_on_any_4_byte_boundary(capi, n_t, off):
+    """FP32 filterbanks whose rows start on any multiple of 4 bytes, with the
+    trials' windows partly and wholly past the end of their rows."""
+    n_chan, n_dm = 64, 40
+    args = (1670.0, 4.0, 64e-6, 20.0, 0.2)
+    delays = O.dm_delays(n_chan, *args, n_dm)
+    plan = capi.DedispPlan(n_chan, n_t, *args, n_dm, n_t)
+    assert plan.info.workspace_bytes > 4 * n_chan * n_dm   # summed by groups
+    fb = S.filterbank_noise(n_chan, n_t, n_t + off)
+    # the samples around the filterbank must not be summed
+    buf = torch.full((n_chan * n_t + 8,), 1e6, device="cuda")
+    view = buf[off:off + n_chan * n_t].view(n_chan, n_t)
+    view.copy_(torch.from_numpy(fb))
+    got = plan.dedisperse(view).cpu().numpy().astype(np.float64)
+    ref = O.dedisperse(fb.astype(np.float64), delays, n_t)
+    bound = O.dedisperse(np.abs(fb.astype(np.float64)), delays, n_t) * (n_chan - 1) * 2.0 ** -24
+    assert np.all(np.abs(got - ref) <= bound + 1e-6)
+    plan.close()
