@@ -511,13 +511,9 @@ static bool bounds_pay(const Plan &p) {
            p.sigma >= (p.H == 16 ? 5.4 : 5.0);
 }
 
-// the workspace of the sums by bounds for these row blocks (none where they
-// do not pay or a harmonic's sources span more than two blocks)
-static fdas_status build_pool(Plan &p, const std::vector<int32_t> &blk) {
-    std::vector<uint32_t> src;
-    std::vector<uint4> masks;
-    if (!bounds_pay(p) || !pool_sources(blk, p.n_z, p.iz0, p.H, &src, &masks)) return FDAS_OK;
-    const int64_t before = p.ws_bytes;
+// the workspace of the sums by bounds for the row blocks `blk`
+static fdas_status alloc_pool(Plan &p, const std::vector<int32_t> &blk,
+                              const std::vector<uint32_t> &src, const std::vector<uint4> &masks) {
     p.pool_nb = (int)blk.size() - 1;
     const int64_t boxes = (int64_t)p.pool_nb * (plane_cols(p) / 2);
     p.pool_list_cap = (unsigned)std::max<int64_t>(4096, boxes / 64);
@@ -532,11 +528,50 @@ static fdas_status build_pool(Plan &p, const std::vector<int32_t> &blk) {
     FDAS_CUDA_TRY(cudaMemcpy(p.pool_src, src.data(), sizeof(uint32_t) * src.size(), cudaMemcpyHostToDevice));
     FDAS_CUDA_TRY(cudaMemcpy(p.pool_masks, masks.data(), sizeof(uint4) * masks.size(),
                              cudaMemcpyHostToDevice));
-    p.pool_bytes = p.ws_bytes - before;
-    p.pool_on = true;
+    // (a copy from pageable memory may return before it has landed)
+    FDAS_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
     return FDAS_OK;
 }
 
+// template half-widths m(z) = 8 + ceil(|z|/2) on the exact grid
+static std::vector<int32_t> half_widths(const Plan &p) {
+    std::vector<int32_t> m(p.n_z);
+    for (int i = 0; i < p.n_z; ++i) {
+        const double az = std::fabs((double)(i - p.iz0)) * p.z_step;
+        m[i] = 8 + (int32_t)std::ceil(az / 2.0 - 1e-9);
+    }
+    return m;
+}
+
+// Sums by bounds for a finished plan, where they pay and a harmonic's sources
+// span no more than two blocks.  Its memory (about 15 % of two 16-bit planes) is
+// allocated after everything that the plan cannot do without, and a device
+// without room for it leaves the plan on the plain kernel.
+static fdas_status add_pool(Plan &p) {
+    if (!bounds_pay(p)) return FDAS_OK;
+    std::vector<int32_t> blk;
+    if (p.correlator == FDAS_CORR_TENSOR) {
+        int win = 0, ks = 0;
+        std::vector<TcChunk> table = tc_chunk_table(p, half_widths(p), &win, &ks);
+        blk = tc_pool_blocks(table, p.n_z);
+    } else {
+        blk = pool_blocks(p.n_z);
+    }
+    std::vector<uint32_t> src;
+    std::vector<uint4> masks;
+    if (!pool_sources(blk, p.n_z, p.iz0, p.H, &src, &masks)) return FDAS_OK;
+    const int64_t before = p.ws_bytes;
+    const std::string last = g_last_error;
+    const fdas_status st = alloc_pool(p, blk, src, masks);
+    p.pool_bytes = p.ws_bytes - before;
+    p.pool_on = st == FDAS_OK;
+    if (!p.pool_on) free_pool(p);
+    if (st != FDAS_ERR_OOM) return st;
+    g_last_error = last;
+    return FDAS_OK;
+}
+
+// (without the workspace of the sums by bounds, which add_pool adds)
 static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_max, double z_step,
                           int32_t seg_len, int32_t n_harm, const fdas_opts *o) {
     FDAS_TRY(fault_args_check(injected_fault()));
@@ -607,14 +642,11 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
     p.interbin = o->interbin != 0;
     for (int s = 0; s < 6; ++s) p.G[s] = s < p.n_stages ? gamma_tail_factor(1 << s, p.sigma) : 0.0;
 
-    // template half-widths m(z) = 8 + ceil(|z|/2) on the exact grid
-    std::vector<int32_t> m(p.n_z);
+    const std::vector<int32_t> m = half_widths(p);
     std::vector<int64_t> off(p.n_z);
     int64_t acc = 0;
     p.m_max = 0;
     for (int i = 0; i < p.n_z; ++i) {
-        const double az = std::fabs((double)(i - p.iz0)) * z_step;
-        m[i] = 8 + (int32_t)std::ceil(az / 2.0 - 1e-9);
         p.m_max = std::max(p.m_max, (int)m[i]);
         off[i] = acc;
         acc += 2 * m[i] + 1;
@@ -727,7 +759,6 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
     // itself and needs only its edge table (allocated below)
     if (p.interbin && p.correlator != FDAS_CORR_TENSOR)
         PLAN_TRY(dalloc(p, &p.corr, cb * (size_t)p.n_z * (size_t)p.n_r, "corr"));
-    PLAN_TRY(build_pool(p, tc_table.empty() ? pool_blocks(p.n_z) : tc_pool_blocks(tc_table, p.n_z)));
     PLAN_TRY(grow_stats(p, 64));
     const int64_t rec_cap = next_pow2(p.max_cands);
     PLAN_TRY(dalloc(p, &p.cand, sizeof(CandRec) * (size_t)rec_cap, "cand"));
@@ -781,6 +812,7 @@ static fdas_status create(Plan *&out, int64_t n_samples, double tsamp, double z_
     PLAN_CUDA(cudaMemcpy(p.tap_m, m.data(), sizeof(int32_t) * p.n_z, cudaMemcpyHostToDevice));
     PLAN_TRY(launch_template_bank(p, p.aux));
     if (p.correlator == FDAS_CORR_TENSOR) {
+        tc_pool_blocks(tc_table, p.n_z);   // the chunks' first row blocks
         const int64_t img = tc_bank_bytes(tc_table);
         PLAN_TRY(dalloc(p, &p.tc_chunks, sizeof(TcChunk) * tc_table.size(), "tc_chunks"));
         if (p.tc_split) {
@@ -1307,8 +1339,7 @@ static fdas_status time_correlation(Plan &p, double &ms) {
 // order (chunk table, template images, shared-memory layout)
 static fdas_status retable_tc(Plan &p, int order) {
     if (p.correlator != FDAS_CORR_TENSOR || p.tc_order == order) return FDAS_OK;
-    std::vector<int32_t> m(p.n_z);
-    FDAS_CUDA_TRY(cudaMemcpy(m.data(), p.tap_m, sizeof(int32_t) * p.n_z, cudaMemcpyDeviceToHost));
+    const std::vector<int32_t> m = half_widths(p);
     const int old_order = p.tc_order, old_win = p.tc_win, old_ks = p.tc_max_ks, old_n = p.tc_n_ch;
     p.tc_order = order;
     std::vector<TcChunk> table = tc_chunk_table(p, m, &p.tc_win, &p.tc_max_ks);
@@ -1321,8 +1352,7 @@ static fdas_status retable_tc(Plan &p, int order) {
         return FDAS_ERR_UNSUPPORTED;
     }
     FDAS_CUDA_TRY(cudaDeviceSynchronize());
-    free_pool(p);   // its row blocks follow the chunks
-    FDAS_TRY(build_pool(p, tc_pool_blocks(table, p.n_z)));
+    tc_pool_blocks(table, p.n_z);   // the chunks' first row blocks
     const int64_t img = tc_bank_bytes(table);
     p.ws_bytes -= p.tc_img_bytes + (int64_t)sizeof(TcChunk) * old_n;
     dfree(p, p.tc_chunks);
@@ -1457,6 +1487,10 @@ fdas_status fdas_plan_create(fdas_plan **out, int64_t n_samples, double tsamp, d
         fdas_status s = o.autotune ? create_tuned(p, n_samples, tsamp, z_max, z_step, seg_len,
                                                   n_harm, o)
                                    : create(p, n_samples, tsamp, z_max, z_step, seg_len, n_harm, &o);
+        if (s == FDAS_OK && (s = add_pool(*p)) != FDAS_OK) {
+            free_plan_memory(p);
+            delete p;
+        }
         if (s == FDAS_OK) *out = reinterpret_cast<fdas_plan *>(p);
         return s;
     } catch (...) {

@@ -147,3 +147,44 @@ def test_every_failed_allocation_frees_the_plan(capi, monkeypatch, prec):
     monkeypatch.delenv("FDAS_FAULT")
     torch.cuda.synchronize()
     assert abs(torch.cuda.mem_get_info()[0] - free0) < (4 << 20)
+
+
+def _same_records(a, b):
+    return a.tobytes() == b.tobytes()
+
+
+@pytest.mark.parametrize("prec,corr", [(0, 1), (1, 2)])
+def test_a_plan_without_room_for_the_bounds_is_created_and_finds_the_same(capi, monkeypatch, prec,
+                                                                         corr):
+    """The workspace of the harmonic sum by bounds is an addition to the plan:
+    where one of its allocations fails the plan holds none of it and sums
+    plainly, and every allocation before it still fails the creation."""
+    make = lambda: capi.Plan(1 << 15, 64e-6, 16.0, 1.0, 2048, 8, precision=prec, correlator=corr)
+    xs = [torch.from_numpy(S.sinusoid_series(n=1 << 15, seed=k, r0=1500.2, z0=2.0, amp=0.3)).cuda()
+          for k in range(3)]
+    plan = make()
+    full = plan.info.workspace_bytes
+    st, ref, n_ref = plan.search(xs)
+    assert st == capi.FDAS_OK and n_ref > 100
+    plan.close()
+    without = set()
+    n_without = 0
+    for k in range(1, 64):
+        monkeypatch.setenv("FDAS_FAULT", f"alloc:{k}")
+        try:
+            plan = make()
+        except capi.FdasError as e:
+            assert e.status == capi.FDAS_ERR_OOM and n_without == 0, (k, e)
+            continue
+        finally:
+            monkeypatch.delenv("FDAS_FAULT")
+        ws = plan.info.workspace_bytes
+        if ws < full:
+            n_without += 1
+            without.add(ws)
+            st, got, n = plan.search(xs)
+            assert st == capi.FDAS_OK and n == n_ref and _same_records(got, ref)
+        plan.close()
+        if ws == full:
+            break
+    assert n_without >= 2 and len(without) == 1 and ws == full
