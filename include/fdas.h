@@ -567,9 +567,9 @@ fdas_status fdas_dedisperse_u8(fdas_dedisp_plan *plan, const uint8_t *filterbank
  *               fdas_plan_create, N >= 1; "alloc" means "alloc:1") fails as
  *               if the device were out of memory: FDAS_ERR_OOM, and a failed
  *               fdas_plan_create frees everything it had allocated.  The
- *               last ones, the workspace of the harmonic sum by bounds, are
- *               optional: the plan is created without it, with the same
- *               results;
+ *               last ones, autotune's other template order and the workspace
+ *               of the harmonic sum by bounds, are optional: the plan is
+ *               created without them, with the same results;
  *   "capacity"  fdas_search / fdas_threshold run with a device candidate
  *               store of one record: two or more crossings give
  *               FDAS_ERR_CAND_STORE_FULL;

@@ -1335,41 +1335,50 @@ static fdas_status time_correlation(Plan &p, double &ms) {
     return FDAS_OK;
 }
 
-// rebuild the tensor-core template chunks of a plan in another template
-// order (chunk table, template images, shared-memory layout)
+// Rebuild the tensor-core template chunks of a plan in another template
+// order (chunk table, template images, shared-memory layout).  The new ones are
+// made in a copy of the plan and take the old ones' place when all of it has
+// succeeded; on an error the plan is as it was.
 static fdas_status retable_tc(Plan &p, int order) {
     if (p.correlator != FDAS_CORR_TENSOR || p.tc_order == order) return FDAS_OK;
-    const std::vector<int32_t> m = half_widths(p);
-    const int old_order = p.tc_order, old_win = p.tc_win, old_ks = p.tc_max_ks, old_n = p.tc_n_ch;
-    p.tc_order = order;
-    std::vector<TcChunk> table = tc_chunk_table(p, m, &p.tc_win, &p.tc_max_ks);
-    if (!tc_applicable(p, nullptr)) {
-        p.tc_order = old_order;
-        p.tc_win = old_win;
-        p.tc_max_ks = old_ks;
-        p.tc_n_ch = old_n;
+    Plan q = p;
+    q.tc_order = order;
+    std::vector<TcChunk> table = tc_chunk_table(q, half_widths(q), &q.tc_win, &q.tc_max_ks);
+    if (!tc_applicable(q, nullptr)) {
         set_error("template order does not fit in shared memory");
         return FDAS_ERR_UNSUPPORTED;
     }
-    FDAS_CUDA_TRY(cudaDeviceSynchronize());
-    tc_pool_blocks(table, p.n_z);   // the chunks' first row blocks
+    tc_pool_blocks(table, q.n_z);   // the chunks' first row blocks
     const int64_t img = tc_bank_bytes(table);
-    p.ws_bytes -= p.tc_img_bytes + (int64_t)sizeof(TcChunk) * old_n;
-    dfree(p, p.tc_chunks);
-    dfree(p, p.tc_bank);
-    p.tc_chunks = nullptr;
-    p.tc_bank = nullptr;
-    FDAS_TRY(dalloc(p, &p.tc_chunks, sizeof(TcChunk) * table.size(), "tc_chunks"));
-    if (p.tc_split) p.tc_bank_lo = img;
-    FDAS_TRY(dalloc(p, &p.tc_bank, (size_t)img * (p.tc_split ? 2 : 1), "tc_bank"));
-    p.tc_img_bytes = img * (p.tc_split ? 2 : 1);
-    p.tc_n_ch = (int)table.size();
-    p.tc_nbuf = tc_image_buffers(p);
-    FDAS_CUDA_TRY(cudaMemcpy(p.tc_chunks, table.data(), sizeof(TcChunk) * table.size(),
-                             cudaMemcpyHostToDevice));
-    FDAS_TRY(launch_tc_bank(p, p.aux));
-    FDAS_CUDA_TRY(cudaStreamSynchronize(p.aux));
-    return FDAS_OK;
+    q.tc_n_ch = (int)table.size();
+    q.tc_nbuf = tc_image_buffers(q);
+    q.tc_img_bytes = img * (q.tc_split ? 2 : 1);
+    if (q.tc_split) q.tc_bank_lo = img;
+    q.tc_chunks = nullptr;
+    q.tc_bank = nullptr;
+    auto build = [&]() -> fdas_status {
+        FDAS_TRY(dalloc(q, &q.tc_chunks, sizeof(TcChunk) * table.size(), "tc_chunks"));
+        FDAS_TRY(dalloc(q, &q.tc_bank, (size_t)q.tc_img_bytes, "tc_bank"));
+        FDAS_CUDA_TRY(cudaMemcpyAsync(q.tc_chunks, table.data(), sizeof(TcChunk) * table.size(),
+                                      cudaMemcpyHostToDevice, q.aux));
+        FDAS_TRY(launch_tc_bank(q, q.aux));
+        FDAS_CUDA_TRY(cudaStreamSynchronize(q.aux));
+        return FDAS_OK;
+    };
+    const fdas_status st = build();
+    if (st == FDAS_OK) {
+        FDAS_CUDA_TRY(cudaDeviceSynchronize());   // nothing reads the old ones any more
+        std::swap(p, q);
+        p.ws_bytes -= q.tc_img_bytes + (int64_t)sizeof(TcChunk) * q.tc_n_ch;
+    } else {
+        // (the templates' energies, which launch_tc_bank writes too, are the same
+        // for every order)
+        cudaStreamSynchronize(q.aux);
+        p.n_allocs = q.n_allocs;
+    }
+    dfree(p, q.tc_chunks);
+    dfree(p, q.tc_bank);
+    return st;
 }
 
 // autotune: the correlator (the tensor-core GEMM, where it applies and was
@@ -1444,11 +1453,10 @@ static fdas_status create_tuned(Plan *&out, int64_t n_samples, double tsamp, dou
         const int first = best->tc_order;
         if (retable_tc(*best, 1 - first) == FDAS_OK) {
             double ms = 0.0;
-            if (time_correlation(*best, ms) == FDAS_OK && ms < best_ms) {
-                best_ms = ms;
-            } else {
-                FDAS_TRY(retable_tc(*best, first));
-            }
+            bool keep = time_correlation(*best, ms) == FDAS_OK && ms < best_ms;
+            // (without room to go back the plan stays in the order it has)
+            if (!keep) keep = retable_tc(*best, first) != FDAS_OK;
+            if (keep) best_ms = ms;
         }
     }
     best->tuned_ms = best_ms;

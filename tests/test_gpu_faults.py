@@ -188,3 +188,35 @@ def test_a_plan_without_room_for_the_bounds_is_created_and_finds_the_same(capi, 
         if ws == full:
             break
     assert n_without >= 2 and len(without) == 1 and ws == full
+
+
+def test_autotune_without_room_for_another_template_order(capi, monkeypatch):
+    """Autotuning a tensor-core plan builds the other template order and may go
+    back; where an allocation of that fails, the plan keeps a whole order (its
+    chunks, images and window belong together) and finds the same cells."""
+    make = lambda **kw: capi.Plan(1 << 14, 64e-6, 60.0, 1.0, 2048, 8, precision=1, correlator=2, **kw)
+    x = torch.from_numpy(S.sinusoid_series(n=1 << 14, seed=3, r0=1500.2, z0=2.0, amp=0.4)).cuda()
+    ref = {}
+    for order in (1, 2):
+        plan = make(template_order=order)
+        assert plan.info.template_order == order
+        st, ref[order], n = plan.search([x])
+        assert st == capi.FDAS_OK and n > 100
+        plan.close()
+    created = 0
+    for k in range(1, 64):
+        monkeypatch.setenv("FDAS_FAULT", f"alloc:{k}")
+        try:
+            plan = make(autotune=True)
+        except capi.FdasError as e:
+            assert e.status == capi.FDAS_ERR_OOM and created == 0, (k, e)
+            continue
+        finally:
+            monkeypatch.delenv("FDAS_FAULT")
+        created += 1
+        want = ref[plan.info.template_order]
+        st, got, n = plan.search([x])
+        assert st == capi.FDAS_OK and n == len(want)
+        assert _same_records(got, want), k
+        plan.close()
+    assert created >= 9   # 2 of the other order, 7 of the bounds' workspace
