@@ -550,7 +550,8 @@ __global__ void __launch_bounds__(Dedup<P, H>::T, 7)
             } else {
                 const float th = st->thr[s];
                 // largest of the 16 sums: they are >= 0, so their bit patterns
-                // order as signed integers (3-input integer max, 8 steps)
+                // order as signed integers (3-input integer max, 8 steps); a NaN
+                // among them is the largest, and the others are compared all the same
                 int mi = __vimax3_s32(__float_as_int(Sv[0].x), __float_as_int(Sv[0].y),
                                       __float_as_int(Sv[1].x));
                 mi = __vimax3_s32(mi, __float_as_int(Sv[1].y), __float_as_int(Sv[2].x));
@@ -559,7 +560,7 @@ __global__ void __launch_bounds__(Dedup<P, H>::T, 7)
                     mi = __vimax3_s32(mi, __float_as_int(Sv[c].y), __float_as_int(Sv[c + 1].x));
                 mi = max(mi, __float_as_int(Sv[D::R / 2 - 1].y));
                 const float m = __int_as_float(mi);
-                if (m * inv > th) {
+                if (!(m * inv <= th)) {
 #pragma unroll
                     for (int i = 0; i < D::R; ++i) {
                         const float val = ((i & 1) ? Sv[i / 2].y : Sv[i / 2].x) * inv;

@@ -111,3 +111,27 @@ def test_a_search_with_many_crossings_and_a_short_series(capi, corr):
         assert _check(capi, sub, plane, mean) == n1
         sub.close()
     plan.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("harm", [2, 8, 16])
+@pytest.mark.parametrize("z_max", [4.0])   # 9 rows: the plain kernel
+def test_cells_beside_nan_and_inf(capi, prec, harm, z_max):
+    """NaN and +inf cells of a caller's plane beside bright ones: the sums that
+    read them are not crossings or are infinite, those beside them (in the same
+    boxes of 2 bins x 4 rows, and through the harmonics) keep their crossings."""
+    plan = capi.Plan(1 << 14, 64e-6, z_max, 1.0, 2048, harm, precision=prec, max_candidates=1 << 22)
+    plane = _plane(plan, 70 + harm)
+    n_z, cols = plane.shape
+    r = np.random.RandomState(harm)
+    scale = 1.0 / 16.0 if prec == 2 else 1.0
+    for k in range(60):
+        z, c = r.randint(1, n_z - 1), r.randint(2, cols - 2)
+        dz, dc = r.randint(-1, 2), r.randint(-1, 2)
+        plane[z, c] = float(r.uniform(60.0, 300.0)) * scale
+        if (dz, dc) != (0, 0):
+            plane[z + dz, c + dc] = float("nan") if k % 4 else float("inf")
+    assert torch.isnan(plane).any() and torch.isinf(plane).any()
+    for mean in (1.0, 0.5):
+        assert _check(capi, plan, plane, mean) > 60
+    plan.close()
