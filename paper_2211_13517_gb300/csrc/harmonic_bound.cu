@@ -23,8 +23,13 @@
 // 17 roundings loses at most 2^-11 of the sum, so the FP16 sum is at least
 // 0.9917 of the true one: thresholds are lowered by 1 % before the
 // comparison.  A threshold outside [0.5, 30000] (a plane far from unit mean)
-// is replaced by 0: every box is then summed exactly.  Cells are powers (>= 0);
-// a NaN never crosses, and max() drops it from the bound of the others.
+// is replaced by 0: every box is then summed exactly.  Cells are powers (>= 0).
+// A cell that is NaN never crosses, and neither does a sum that reads it, but the
+// sums beside it may, so no maximum of a caller's plane is NaN: where pool_kernel
+// compares 16-bit cells as integers a NaN would be the largest, and it becomes
+// +inf there, which sends its box to the exact sums (FP32 maxima drop it).  A plane
+// of the search with a NaN cell has a NaN mean and thresholds that nothing
+// crosses, so the tensor-core epilogue's maxima are left as they are.
 //
 // Bound of the kernel: instruction issue and the latency of the span copies
 // (the gathers move 1/8 of the cells' bytes).
@@ -72,9 +77,11 @@ __global__ void __launch_bounds__(256) pool_kernel(const typename P::real *__res
             m.w = __vmaxs2(m.w, w[r].w);
         }
         const uint32_t mm[4] = {m.x, m.y, m.z, m.w};
+        constexpr uint32_t inf = P::id == FDAS_BF16 ? 0x7f80u : 0x7c00u;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const unsigned short h = (unsigned short)max(mm[k] & 0xffffu, mm[k] >> 16);
+            const unsigned short h =
+                (unsigned short)min(max(mm[k] & 0xffffu, mm[k] >> 16), inf);   // NaN: +inf
             typename P::real v;
             memcpy(&v, &h, 2);
             e[k] = P::ldr(v) * (1.0f / P::plane_scale);

@@ -115,7 +115,7 @@ def test_a_search_with_many_crossings_and_a_short_series(capi, corr):
 
 @pytest.mark.parametrize("prec", [0, 1, 2])
 @pytest.mark.parametrize("harm", [2, 8, 16])
-@pytest.mark.parametrize("z_max", [4.0])   # 9 rows: the plain kernel
+@pytest.mark.parametrize("z_max", [4.0, 96.0])   # 9 rows: the plain kernel; 193: by bounds
 def test_cells_beside_nan_and_inf(capi, prec, harm, z_max):
     """NaN and +inf cells of a caller's plane beside bright ones: the sums that
     read them are not crossings or are infinite, those beside them (in the same
