@@ -468,7 +468,8 @@ fdas_status fdas_spectrum_static(const float *series, int64_t n_samples,
  * series runs on a second stream beside the next series), so that each
  * event interval holds one group's kernels only.
  * Groups: [0] R2C FFT + normalisation, [1] fused correlation/power,
- * [2] statistics + harmonic sum/threshold, [3] candidate ordering/output.
+ * [2] statistics + harmonic sum/threshold, [3] the counters' reset before a
+ * search and the candidate ordering/output after it.
  * --------------------------------------------------------------------- */
 enum { FDAS_PROF_SPECTRUM = 0, FDAS_PROF_CORRELATE = 1, FDAS_PROF_HARMONIC = 2,
        FDAS_PROF_FINISH = 3 };

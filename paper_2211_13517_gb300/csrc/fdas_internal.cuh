@@ -330,6 +330,7 @@ fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, bool 
                                       const TrialStats *st, uint32_t rank,
                                       cudaStream_t s);
 bool sums_by_bounds(const Plan &p);   // whether launch_harmonic_threshold goes by bounds
+int harmonic_launches(const Plan &p, bool pooled);   // and its number of kernels
 // the same crossings from bounds on boxes of cells (pool_on plans)
 constexpr int kPoolMaxRows = 4;   // rows of a block
 std::vector<int32_t> pool_blocks(int n_z);

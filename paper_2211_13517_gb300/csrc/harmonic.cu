@@ -1125,6 +1125,12 @@ fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partia
 
 bool sums_by_bounds(const Plan &p) { return p.pool_on && p.n_r >= kBoundMinCols; }
 
+// by bounds: the pooling unless done, the bounds, the exact sums, and the gated
+// plain kernel
+int harmonic_launches(const Plan &p, bool pooled) {
+    return sums_by_bounds(p) ? (pooled ? 3 : 4) : 1;
+}
+
 fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, bool pooled,
                                       const TrialStats *st, uint32_t rank, cudaStream_t s) {
     const bool by_bounds = sums_by_bounds(p);
@@ -1210,6 +1216,7 @@ fdas_status launch_init_search(Plan &p, const uint32_t *ids, int n, cudaStream_t
     }
     init_search_kernel<<<1, 32, 0, s>>>(arg, n <= 32 ? n : 0, p.rank_ids, p.cand_count, p.flags);
     FDAS_CUDA_TRY(cudaGetLastError());
+    p.launches[FDAS_PROF_FINISH] += 1;
     return FDAS_OK;
 }
 

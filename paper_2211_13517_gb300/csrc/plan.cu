@@ -1128,7 +1128,7 @@ static fdas_status enqueue_batch(Plan &p, const fdas_series *batch, int32_t n_se
         if (hs != s) FDAS_CUDA_TRY(cudaEventRecord(p.ev_hsum[b], hs));
         p.launches[FDAS_PROF_SPECTRUM] += (v.fft_m1 == 1 ? 1 : 2) + 1;
         p.launches[FDAS_PROF_CORRELATE] += p.interbin ? 2 : 1;   // + fix-up or interbinning
-        p.launches[FDAS_PROF_HARMONIC] += 2;
+        p.launches[FDAS_PROF_HARMONIC] += 1 + harmonic_launches(hv, pooled);   // 1: statistics
         if (p.profiling) {
             iv.push_back({FDAS_PROF_SPECTRUM, e0, e1});
             iv.push_back({FDAS_PROF_CORRELATE, e1, e2});
