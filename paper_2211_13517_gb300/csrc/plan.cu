@@ -495,20 +495,39 @@ static Plan plan_view(const Plan &p, int64_t n) {
     return v;
 }
 
-// Whether the harmonic sum goes by bounds (harmonic_bound.cu).  It adds the
-// pooled plane and two kernels, and pays when few bounds reach a threshold and
-// the plane is more than a few rows.  A BF16 search of 2^22 samples x 193 rows
-// (whole call, us; by the plain kernel in brackets, measured with the rule
-// switched): 16 harmonics, 6 sigma 504 (1029), 5.5 sigma 591 (1038), 5 sigma
-// longer by bounds than plain (1138 against 1072 when the rule was set); 8
-// harmonics, 6 sigma 417 (771), 5 sigma 440 (800), 4.5 sigma even then (1004,
-// 998).  One harmonic only compares cells (308 against 288), and with one row
-// the extra launches cost 10 to 15 us.  Unnormalised planes and the mean + k
-// sigma rule (far lower thresholds) keep the plain kernel.
+// Whether the thresholds let the harmonic sum go by bounds (harmonic_bound.cu).
+// It pays as long as noise alone does not overflow the list of boxes (1 box in
+// 64), after which the plain kernel runs as well: a call is then about 25 %
+// longer than by the plain kernel alone.  Neighbouring rows differ more the
+// larger z_step is, and boxes of 4 rows pass more often, so the threshold rises
+// with it.  Plain kernel's time over that by bounds, two noise series of 2^22
+// samples, |z| <= 96 (whole searches; FP32, BF16):
+//
+//   16 harmonics    5.4 sigma   5.75        6           6.5         7
+//   z_step 1        1.29, 1.48  1.41, 1.74  1.45, 1.86  1.48, 1.95  1.49, 1.97
+//   z_step 1.5      0.80, 1.04  1.24, 1.37  1.33, 1.53  1.42, 1.69  1.42, 1.72
+//   z_step 2        0.80, 0.81  0.80, 1.11  1.20, 1.29  1.34, 1.50  1.36, 1.58
+//   z_step 4        0.79, 0.80  0.79, 0.81  0.79, 0.81  1.12, 1.14  1.23, 1.31
+//   z_step 8        0.80, 0.83  0.80, 0.82  0.79, 0.85  0.79, 0.86  1.14, 1.12
+//   8 harmonics     4.5 sigma   5           5.4         6
+//   z_step 1        1.12, 1.30  1.19, 1.54  1.21, 1.63  1.21, 1.66
+//   z_step 2        0.78, 0.91  1.08, 1.24  1.12, 1.33  1.14, 1.38
+//   z_step 4        0.80, 0.82  1.00, 1.01  1.07, 1.13  1.09, 1.21
+//   z_step 8        0.81, 0.87  0.82, 0.85  1.03, 1.04  1.07, 1.13
+//   2 and 4 harmonics, 5 sigma, z_step 1 to 8: 1.01 to 1.09, 1.07 to 1.46
+//
+// On the lines themselves (z_step 1, 1.25, 1.5, ..., 8): 16 harmonics 1.14 to
+// 1.29, 1.11 to 1.45; 8 harmonics 1.00 to 1.19, 1.02 to 1.49.  Periodic signals
+// list boxes of their own, but far fewer than the crossings that they take from
+// the plain kernel (1.2 to 2.8 with 23000 to 9 million crossings).  One harmonic
+// only compares cells (308 us by bounds against 288).  Unnormalised planes and the
+// mean + k sigma rule (far lower thresholds) keep the plain kernel.
 static bool bounds_pay(const Plan &p) {
+    const double octaves = std::log2(std::max(1.0, p.z_step));
+    const double sigma = p.H == 16 ? 5.4 + 0.6 * octaves : p.H == 8 ? 5.0 + 0.125 * octaves : 5.0;
     return p.harm_mode == FDAS_HARM_TOP && p.H >= 2 && p.H <= 16 && p.n_z >= 12 &&
            p.norm_mode == FDAS_NORM_MEDIAN && p.thr_mode == FDAS_THRESH_GAMMA_TAIL &&
-           p.sigma >= (p.H == 16 ? 5.4 : 5.0);
+           p.z_step <= 8.0 && p.sigma >= sigma - 1e-9;
 }
 
 // the workspace of the sums by bounds for the row blocks `blk`

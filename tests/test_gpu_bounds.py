@@ -135,3 +135,43 @@ def test_cells_beside_nan_and_inf(capi, prec, harm, z_max):
     for mean in (1.0, 0.5):
         assert _check(capi, plan, plane, mean) > 60
     plan.close()
+
+
+def _by_bounds(capi, plan):
+    """Whether a search on the plan sums by bounds: by its launches of the harmonic
+    group (2 plain, statistics included)."""
+    plan.profile(False)
+    plan.search([torch.randn(plan.info.n_samples, device="cuda")], capacity=1 << 16)
+    return plan.profile()["harmonic"][0] > 2
+
+
+@pytest.mark.parametrize("harm,z_step,sigma,by_bounds", [
+    (16, 1.0, 5.3, False), (16, 1.0, 5.4, True), (16, 0.5, 5.4, True),
+    (16, 2.0, 5.9, False), (16, 2.0, 6.0, True),
+    (16, 4.0, 6.0, False), (16, 4.0, 6.5, False), (16, 4.0, 6.6, True),
+    (16, 8.0, 7.1, False), (16, 8.0, 7.2, True), (16, 9.0, 8.0, False),
+    (8, 1.0, 4.9, False), (8, 1.0, 5.0, True), (8, 2.0, 5.1, False), (8, 2.0, 5.125, True),
+    (8, 8.0, 5.3, False), (8, 8.0, 5.375, True),
+    (4, 8.0, 4.9, False), (4, 8.0, 5.0, True), (2, 4.0, 5.0, True), (1, 1.0, 6.0, False),
+])
+def test_thresholds_that_go_by_bounds(capi, harm, z_step, sigma, by_bounds):
+    """Where noise alone would overflow the list of boxes the plain kernel is kept."""
+    plan = capi.Plan(1 << 14, 64e-6, 16 * z_step, z_step, 2048, harm, threshold_sigma=sigma)
+    assert _by_bounds(capi, plan) == by_bounds
+    plan.close()
+
+
+@pytest.mark.parametrize("prec,corr", [(0, 1), (1, 2), (2, 2)])
+@pytest.mark.parametrize("z_step,sigma", [(0.5, 5.4), (1.0, 5.4), (2.0, 6.0), (4.0, 6.6), (8.0, 7.2)])
+def test_coarse_and_fine_drift_steps_at_their_lowest_threshold(capi, prec, corr, z_step, sigma):
+    """The plane of a pulse train, 16 harmonics: the crossings by bounds are the plain sums'."""
+    n = 1 << 17
+    plan = capi.Plan(n, 64e-6, 24 * z_step, z_step, 4096, 16, precision=prec, correlator=corr,
+                     threshold_sigma=sigma)
+    assert _by_bounds(capi, plan)
+    u = np.arange(n) / n
+    ph = 1700.3 * u + 2.0 * z_step * (u - 0.5) ** 2
+    x = np.random.RandomState(4).randn(n) + 1.2 * ((ph - np.floor(ph)) < 0.05)
+    plane, stats = plan.power_plane(plan.spectrum(torch.from_numpy(x.astype(np.float32)).cuda()))
+    assert _check(capi, plan, plane, float(stats[0])) > 20
+    plan.close()
