@@ -329,7 +329,8 @@ fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partia
 fdas_status launch_harmonic_threshold(Plan &p, const void *plane, int buf, bool pooled,
                                       const TrialStats *st, uint32_t rank,
                                       cudaStream_t s);
-bool sums_by_bounds(const Plan &p);   // whether launch_harmonic_threshold goes by bounds
+// whether launch_harmonic_threshold goes by bounds (the rule stands in plan.cu)
+bool sums_by_bounds(const Plan &p);
 int harmonic_launches(const Plan &p, bool pooled);   // and its number of kernels
 // the same crossings from bounds on boxes of cells (pool_on plans)
 constexpr int kPoolMaxRows = 4;   // rows of a block

@@ -1105,9 +1105,6 @@ fdas_status launch_hs_P(Plan &p, const void *plane, const TrialStats *st, uint32
     }
 }
 
-// shortest row the bound kernels take
-constexpr int64_t kBoundMinCols = 1 << 11;
-
 }  // namespace
 
 fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partials,
@@ -1122,8 +1119,6 @@ fdas_status launch_finalize_stats(Plan &p, const double2 *partials, int n_partia
     FDAS_CUDA_TRY(cudaGetLastError());
     return FDAS_OK;
 }
-
-bool sums_by_bounds(const Plan &p) { return p.pool_on && p.n_r >= kBoundMinCols; }
 
 // by bounds: the pooling unless done, the bounds, the exact sums, and the gated
 // plain kernel

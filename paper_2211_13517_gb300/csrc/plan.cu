@@ -530,6 +530,45 @@ static bool bounds_pay(const Plan &p) {
            p.z_step <= 8.0 && p.sigma >= sigma - 1e-9;
 }
 
+// And whether a plane of `cols` columns is large enough: few rows and harmonics
+// save less than the pooled plane, two more kernels and the bound kernel's barely
+// filled grid cost.  Plain kernel's time over that by bounds, one noise series,
+// z_step 1, 6 sigma:
+//
+//                   rows    2^16   2^18   2^20   2^21   2^22   2^23 samples
+//   FP32, H = 2      13     0.99   0.98   0.98   0.98   0.98   1.00
+//                    17     1.01   1.04   0.98   1.01   1.00   0.99
+//   FP32, H = 4      13     0.98   0.99   0.99   0.98   0.97   1.00
+//                    17     1.00   1.03   1.04   1.01   0.99   1.00
+//   FP32, H = 8      13     1.01   0.99   0.97   0.99   1.08   1.04
+//                    15     1.06   1.01   1.00   1.02   1.10   1.05
+//   FP32, H = 16     13     0.97   0.98   0.97   1.13   1.15   1.17
+//                    15     1.00   1.00   1.02   1.16   1.19   1.19
+//   16-bit, H = 2    17     1.02   0.99   0.98   0.96   0.93   1.01
+//                    25     1.03   1.00   0.96   0.95   0.99   1.07
+//                    49     1.00   1.00   0.95   1.06   1.11
+//                    97     1.02   1.01   1.07   1.14   1.22
+//   16-bit, H = 4    17     1.02   0.99   0.98   0.99   0.92   0.98
+//                    25     1.02   1.00   1.02   0.99   1.00   1.07
+//                    49     1.01   1.00   0.98   1.06   1.07
+//                    97     1.01   1.02   1.09   1.13   1.23
+//   16-bit, H = 8    15     1.01   0.98   0.98   0.99   0.96   1.00
+//                    17     1.06   1.02   1.03   1.01   0.96   1.01
+//                    25     1.04   1.03   1.01   0.97   1.03   1.12
+//   16-bit, H = 16   13     0.99   0.98   1.01   1.00   0.98   1.04
+//                    15     1.02   1.01   1.03   1.01   1.00   1.07
+static bool bounds_pay_at(const Plan &p, int64_t cols) {
+    if (cols < 1 << 11) return false;   // the bound kernel's columns of boxes
+    const int64_t cells = p.n_z * cols;
+    if (p.prec == FDAS_FP32)
+        return p.n_z >= 15 || (p.H >= 8 && cells >= (p.H == 16 ? 8 << 20 : 16 << 20));
+    if (p.H <= 4) return p.n_z >= 24 && cells >= 48 << 20;
+    if (p.H == 8) return p.n_z >= 24 || (p.n_z >= 16 && (cells <= 4 << 20 || cells >= 64 << 20));
+    return p.n_z >= 15 || cells >= 48 << 20;
+}
+
+bool sums_by_bounds(const Plan &p) { return p.pool_on && bounds_pay_at(p, p.n_r); }
+
 // the workspace of the sums by bounds for the row blocks `blk`
 static fdas_status alloc_pool(Plan &p, const std::vector<int32_t> &blk,
                               const std::vector<uint32_t> &src, const std::vector<uint4> &masks) {
@@ -567,7 +606,9 @@ static std::vector<int32_t> half_widths(const Plan &p) {
 // allocated after everything that the plan cannot do without, and a device
 // without room for it leaves the plan on the plain kernel.
 static fdas_status add_pool(Plan &p) {
-    if (!bounds_pay(p)) return FDAS_OK;
+    bool any = false;   // series may be shorter than the plan's
+    for (int64_t cols = plane_cols(p); cols >= 1 << 9; cols /= 2) any = any || bounds_pay_at(p, cols);
+    if (!any || !bounds_pay(p)) return FDAS_OK;
     std::vector<int32_t> blk;
     if (p.correlator == FDAS_CORR_TENSOR) {
         int win = 0, ks = 0;

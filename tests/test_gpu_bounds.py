@@ -175,3 +175,32 @@ def test_coarse_and_fine_drift_steps_at_their_lowest_threshold(capi, prec, corr,
     plane, stats = plan.power_plane(plan.spectrum(torch.from_numpy(x.astype(np.float32)).cuda()))
     assert _check(capi, plan, plane, float(stats[0])) > 20
     plan.close()
+
+
+@pytest.mark.parametrize("prec,harm,n_log2,rows,by_bounds", [
+    (0, 16, 14, 13, False), (0, 16, 14, 15, True), (0, 16, 21, 13, True), (0, 8, 21, 13, False),
+    (0, 8, 22, 13, True), (0, 2, 22, 13, False), (0, 2, 14, 15, True), (0, 16, 11, 27, False),
+    (0, 16, 12, 27, True), (0, 16, 22, 11, False),
+    (1, 16, 14, 13, False), (1, 16, 14, 15, True), (1, 8, 14, 15, False), (1, 8, 14, 17, True),
+    (1, 8, 20, 23, False), (1, 8, 20, 25, True), (1, 8, 23, 17, True), (1, 4, 20, 95, False),
+    (1, 4, 20, 97, True), (2, 2, 18, 193, False), (2, 2, 23, 23, False),
+])
+def test_sizes_that_go_by_bounds(capi, prec, harm, n_log2, rows, by_bounds):
+    plan = capi.Plan(1 << n_log2, 64e-6, float(rows // 2), 1.0, 2048 if n_log2 > 11 else 1024, harm,
+                     precision=prec)
+    assert plan.info.n_z == rows
+    assert _by_bounds(capi, plan) == by_bounds
+    plan.close()
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("harm", [2, 4])
+def test_few_harmonics_of_a_large_plane(capi, prec, harm):
+    plan = capi.Plan(1 << 20, 64e-6, 48.0, 1.0, 2048, harm, precision=prec, threshold_sigma=5.0)
+    assert _by_bounds(capi, plan)
+    u = np.arange(1 << 20) / (1 << 20)
+    ph = 17000.3 * u + 2.0 * (u - 0.5) ** 2
+    x = np.random.RandomState(4).randn(1 << 20) + 0.4 * ((ph - np.floor(ph)) < 0.05)
+    plane, stats = plan.power_plane(plan.spectrum(torch.from_numpy(x.astype(np.float32)).cuda()))
+    assert _check(capi, plan, plane, float(stats[0])) > 20
+    plan.close()
