@@ -888,7 +888,7 @@ template <class P, int H, bool kWriteSums>
 fdas_status launch_hs(Plan &p, const void *plane, const TrialStats *st, uint32_t rank,
                       float *sums_out, bool gated, cudaStream_t s) {
     if constexpr (H <= 16) {
-        if constexpr (!kWriteSums)
+        if constexpr (!kWriteSums && H >= 2)   // one harmonic never goes by bounds
             if (gated) return launch_dedup<P, H, false, true>(p, plane, st, rank, nullptr, s);
         return launch_dedup<P, H, kWriteSums, false>(p, plane, st, rank, sums_out, s);
     }

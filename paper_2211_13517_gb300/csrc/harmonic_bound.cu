@@ -555,7 +555,6 @@ fdas_status launch_bound_P(Plan &p, const void *plane, int buf, bool pooled, con
         FDAS_CUDA_TRY(cudaGetLastError());
     }
     switch (p.H) {
-        case 1: return launch_bound<P, 1>(p, plane, buf, st, rank, s);
         case 2: return launch_bound<P, 2>(p, plane, buf, st, rank, s);
         case 4: return launch_bound<P, 4>(p, plane, buf, st, rank, s);
         case 8: return launch_bound<P, 8>(p, plane, buf, st, rank, s);
