@@ -204,3 +204,71 @@ def test_few_harmonics_of_a_large_plane(capi, prec, harm):
     plane, stats = plan.power_plane(plan.spectrum(torch.from_numpy(x.astype(np.float32)).cuda()))
     assert _check(capi, plan, plane, float(stats[0])) > 20
     plan.close()
+
+
+def _sparse_plane(plan, seed):
+    """Cells below 0.5, whose sums cross nothing and list no box, and 8 bright ones,
+    among them the corners: less than 300 boxes read one, so the list (4096 boxes at
+    least) never overflows."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    shape = (plan.info.n_z, plan.info.plane_cols)
+    p = 0.5 * torch.rand(shape, generator=g, device="cuda")
+    r = np.random.RandomState(seed)
+    for _ in range(4):
+        p[r.randint(shape[0]), r.randint(shape[1])] = float(r.uniform(60.0, 300.0))
+    p[0, 0] = p[-1, -1] = p[0, -1] = p[-1, 0] = 60.0
+    return (p / 16.0 if plan.info.precision == 2 else p).to(plan.spec_dtype)
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("harm", [8, 16])
+@pytest.mark.parametrize("n_log2,rows,by_bounds", [(11, 27, False), (12, 25, True), (12, 27, True),
+                                                   (13, 29, True), (14, 193, True)])
+def test_a_few_bright_cells(capi, prec, harm, n_log2, rows, by_bounds):
+    """By bounds and the exact sums alone, at the shortest rows (1024 columns are too
+    few) and where the last block of rows and the last step of 8 blocks are partial;
+    with every threshold out of FP16's range; and with every cell a crossing, which
+    overflows the list of any plane of more than 4096 boxes."""
+    plan = capi.Plan(1 << n_log2, 64e-6, float(rows // 2), 1.0, 2048 if n_log2 > 11 else 1024, harm,
+                     precision=prec, max_candidates=1 << 23)
+    assert plan.info.n_z == rows and _by_bounds(capi, plan) == by_bounds
+    plane = _sparse_plane(plan, rows + harm)
+    assert _check(capi, plan, plane, 1.0) >= 8
+    for scale in (1e-3, 1e4):
+        assert _check(capi, plan, plane * scale, scale) >= 8
+    if n_log2 <= 13:
+        full = torch.full_like(plane, 40.0 / (16.0 if prec == 2 else 1.0))
+        assert _check(capi, plan, full, 1.0) == full.numel() * plan.info.n_stages
+    plan.close()
+
+
+@pytest.mark.parametrize("prec,corr,interbin", [(1, 2, False), (2, 2, False), (0, 3, False),
+                                                (1, 2, True), (2, 2, True), (0, 1, True)])
+def test_pooled_planes_of_the_correlation_and_of_the_plane(capi, prec, corr, interbin):
+    """A search, whose pooled plane the tensor-core epilogue writes (with half bins the
+    fix-up kernel too), against fdas_threshold on the same plane, which pools it by a
+    kernel, and against the plain sums; a series of the plan's length and a half of it."""
+    import synthetic as S
+    n = 1 << 15
+    make = lambda m: capi.Plan(m, 64e-6, 30.0, 1.0, 2048, 16, precision=prec, correlator=corr,
+                               interbin=interbin)
+    plan = make(n)
+    assert _by_bounds(capi, plan)
+    for m in (n, n // 2):
+        # a tone half-way between two bins, the last one of its warp
+        x = S.inject_sinusoid(S.white_noise(m, 7), 255.5 + 512 * (m // 2048), 2.0, 0.5)
+        x = torch.from_numpy(x).cuda()
+        st, found, nf = plan.search([x], capacity=1 << 18)
+        assert st == capi.FDAS_OK and nf == len(found) > 100
+        sub = make(m)
+        plane, stats = sub.power_plane(sub.spectrum(x))
+        st, staged, _ = sub.threshold(plane, stats, capacity=1 << 18)
+        # (not sigma: the fix-up kernel sums the half bins' statistics by row blocks in a
+        # search, by rows in a stage call, and their means differ by FP32 rounding)
+        assert st == capi.FDAS_OK and len(found) == len(staged)
+        for k in ("harm", "iz", "ir", "power"):
+            assert np.array_equal(found[k], staged[k]), k
+        assert _check(capi, sub, plane, float(stats[0])) == nf
+        sub.close()
+    plan.close()
