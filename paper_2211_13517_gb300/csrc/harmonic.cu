@@ -498,90 +498,90 @@ __global__ void __launch_bounds__(Dedup<P, H>::T, 7)
     const int cols = (int)((n_r + D::CELLS - 1) / D::CELLS);
     const int n_tiles = cols * ((n_z + D::QROWS - 1) / D::QROWS);
     for (int tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x) {
-    const int64_t B = (int64_t)(tile % cols) * D::CELLS;
-    const int iz_begin = tile / cols * D::QROWS;
-    const int iz_end = min(iz_begin + D::QROWS, n_z);
-    const int64_t b = B + (int64_t)D::R * t;   // first cell of this thread
-    const bool active = b < n_r;   // thread 0 always is
-    uint32_t tv[8];   // 16-bit planes: the thread's top-row cells, one row ahead
-    if constexpr (D::kTopRegs)
-        if (active && iz_begin < iz_end &&
-            FDAS_IN_BOUNDS((int64_t)iz_begin * n_r + b, D::R, (int64_t)n_z * n_r, kSiteHsTopLoad))
-            Steps::load_top(plane + (int64_t)iz_begin * n_r + b, tv);
-    for (int iz = iz_begin; iz < iz_end; ++iz, ++q) {
-        // every thread is done with the previous row's spans (and, for the
-        // first row, the barriers are initialised); stop together after a
-        // wait that gave up
-        if (__syncthreads_or(failed)) {
-            failed = true;
-            break;
-        }
-        if (t < 32) {
-            // the spans whose source row changed, over the previous row's
-            // (their reads by this CTA's threads come before the copies),
-            // then one arrival per stage barrier (none on the unused barrier
-            // of a top row held in registers)
-            Steps::copy_lane(lane_sp, plane, iz0, iz - iz0, n_r, B, iz == iz_begin, sm,
-                             bars, n_z);
-            __syncwarp();
-            if (t < Steps::NG && !(t == 0 && D::kTopRegs)) mbar_arrive(&bars[t]);
-        }
-        if (!active) continue;
-        float2 S2[D::R / 2];
+        const int64_t B = (int64_t)(tile % cols) * D::CELLS;
+        const int iz_begin = tile / cols * D::QROWS;
+        const int iz_end = min(iz_begin + D::QROWS, n_z);
+        const int64_t b = B + (int64_t)D::R * t;   // first cell of this thread
+        const bool active = b < n_r;   // thread 0 always is
+        uint32_t tv[8];   // 16-bit planes: the thread's top-row cells, one row ahead
+        if constexpr (D::kTopRegs)
+            if (active && iz_begin < iz_end &&
+                FDAS_IN_BOUNDS((int64_t)iz_begin * n_r + b, D::R, (int64_t)n_z * n_r, kSiteHsTopLoad))
+                Steps::load_top(plane + (int64_t)iz_begin * n_r + b, tv);
+        for (int iz = iz_begin; iz < iz_end; ++iz, ++q) {
+            // every thread is done with the previous row's spans (and, for the
+            // first row, the barriers are initialised); stop together after a
+            // wait that gave up
+            if (__syncthreads_or(failed)) {
+                failed = true;
+                break;
+            }
+            if (t < 32) {
+                // the spans whose source row changed, over the previous row's
+                // (their reads by this CTA's threads come before the copies),
+                // then one arrival per stage barrier (none on the unused barrier
+                // of a top row held in registers)
+                Steps::copy_lane(lane_sp, plane, iz0, iz - iz0, n_r, B, iz == iz_begin, sm,
+                                 bars, n_z);
+                __syncwarp();
+                if (t < Steps::NG && !(t == 0 && D::kTopRegs)) mbar_arrive(&bars[t]);
+            }
+            if (!active) continue;
+            float2 S2[D::R / 2];
 #pragma unroll
-        for (int c = 0; c < D::R / 2; ++c) S2[c] = make_float2(0.f, 0.f);
-        const real *next_top =
-            iz + 1 < iz_end && FDAS_IN_BOUNDS((int64_t)(iz + 1) * n_r + b, D::R,
-                                              (int64_t)n_z * n_r, kSiteHsTopLoad)
-                ? plane + (int64_t)(iz + 1) * n_r + b
-                : nullptr;
-        const bool ok = Steps::template sums<0>(sm, bars, (unsigned)(q & 1), t, S2,
-                                                [&](int s, float2 (&Sv)[D::R / 2]) {
-            if constexpr (kWriteSums) {
-                if (!FDAS_IN_BOUNDS(((int64_t)s * n_z + iz) * n_r + b, D::R,
-                                    (int64_t)(ilog2h(H) + 1) * n_z * n_r, kSiteHsSumsStore))
-                    return;
+            for (int c = 0; c < D::R / 2; ++c) S2[c] = make_float2(0.f, 0.f);
+            const real *next_top =
+                iz + 1 < iz_end && FDAS_IN_BOUNDS((int64_t)(iz + 1) * n_r + b, D::R,
+                                                  (int64_t)n_z * n_r, kSiteHsTopLoad)
+                    ? plane + (int64_t)(iz + 1) * n_r + b
+                    : nullptr;
+            const bool ok = Steps::template sums<0>(sm, bars, (unsigned)(q & 1), t, S2,
+                                                    [&](int s, float2 (&Sv)[D::R / 2]) {
+                if constexpr (kWriteSums) {
+                    if (!FDAS_IN_BOUNDS(((int64_t)s * n_z + iz) * n_r + b, D::R,
+                                        (int64_t)(ilog2h(H) + 1) * n_z * n_r, kSiteHsSumsStore))
+                        return;
 #pragma unroll
-                for (int c = 0; c < D::R / 2; ++c) {
-                    float *o = sums_out + ((int64_t)s * n_z + iz) * n_r + b + 2 * c;
-                    o[0] = Sv[c].x * inv;
-                    o[1] = Sv[c].y * inv;
-                }
-            } else {
-                const float th = st->thr[s];
-                // largest of the 16 sums: they are >= 0, so their bit patterns
-                // order as signed integers (3-input integer max, 8 steps); a NaN
-                // among them is the largest, and the others are compared all the same
-                int mi = __vimax3_s32(__float_as_int(Sv[0].x), __float_as_int(Sv[0].y),
-                                      __float_as_int(Sv[1].x));
-                mi = __vimax3_s32(mi, __float_as_int(Sv[1].y), __float_as_int(Sv[2].x));
+                    for (int c = 0; c < D::R / 2; ++c) {
+                        float *o = sums_out + ((int64_t)s * n_z + iz) * n_r + b + 2 * c;
+                        o[0] = Sv[c].x * inv;
+                        o[1] = Sv[c].y * inv;
+                    }
+                } else {
+                    const float th = st->thr[s];
+                    // largest of the 16 sums: they are >= 0, so their bit patterns
+                    // order as signed integers (3-input integer max, 8 steps); a NaN
+                    // among them is the largest, and the others are compared all the same
+                    int mi = __vimax3_s32(__float_as_int(Sv[0].x), __float_as_int(Sv[0].y),
+                                          __float_as_int(Sv[1].x));
+                    mi = __vimax3_s32(mi, __float_as_int(Sv[1].y), __float_as_int(Sv[2].x));
 #pragma unroll
-                for (int c = 2; c < D::R / 2 - 1; ++c)
-                    mi = __vimax3_s32(mi, __float_as_int(Sv[c].y), __float_as_int(Sv[c + 1].x));
-                mi = max(mi, __float_as_int(Sv[D::R / 2 - 1].y));
-                const float m = __int_as_float(mi);
-                if (!(m * inv <= th)) {
+                    for (int c = 2; c < D::R / 2 - 1; ++c)
+                        mi = __vimax3_s32(mi, __float_as_int(Sv[c].y), __float_as_int(Sv[c + 1].x));
+                    mi = max(mi, __float_as_int(Sv[D::R / 2 - 1].y));
+                    const float m = __int_as_float(mi);
+                    if (!(m * inv <= th)) {
 #pragma unroll
-                    for (int i = 0; i < D::R; ++i) {
-                        const float val = ((i & 1) ? Sv[i / 2].y : Sv[i / 2].x) * inv;
-                        if (val > th) {
-                            const unsigned long long idx = atomicAdd(count, 1ull);
-                            if ((int64_t)idx < cap) {
-                                CandRec rec;
-                                rec.key = cand_key(rank, s, iz, (uint32_t)(b + i));
-                                rec.power = val;
-                                rec.pad = 0.f;
-                                cand[idx] = rec;
+                        for (int i = 0; i < D::R; ++i) {
+                            const float val = ((i & 1) ? Sv[i / 2].y : Sv[i / 2].x) * inv;
+                            if (val > th) {
+                                const unsigned long long idx = atomicAdd(count, 1ull);
+                                if ((int64_t)idx < cap) {
+                                    CandRec rec;
+                                    rec.key = cand_key(rank, s, iz, (uint32_t)(b + i));
+                                    rec.power = val;
+                                    rec.pad = 0.f;
+                                    cand[idx] = rec;
+                                }
                             }
                         }
                     }
                 }
-            }
-        }, tv, next_top);
-        if (!ok) failed = true;
-    }
-    failed = __syncthreads_or(failed);
-    if constexpr (!kGated) break;   // one tile per CTA
+            }, tv, next_top);
+            if (!ok) failed = true;
+        }
+        failed = __syncthreads_or(failed);
+        if constexpr (!kGated) break;   // one tile per CTA
     }
     if (failed) {
         if (t == 0) atomicOr(flags, 2u);
