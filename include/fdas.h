@@ -516,7 +516,10 @@ fdas_status fdas_selftest_wait_timeout(fdas_plan *plan, int64_t limit_cycles, vo
  * that order (f_c, 1/f_c^2, 1/f_top^2, DM_d, (K DM_d)(a - b), / tsamp,
  * + 1/2, floor), and the series is
  *   out[d][t] = sum_{c} in[c][t + Delta(c, d)],  t < n_out,
- * with samples at or past n_t counted as 0 (FP32 sums in channel order).
+ * with samples at or past n_t counted as 0.  FP32 sums, in channel order or
+ * of up to 4 neighbouring channels at a time (where their delays take few
+ * patterns; the plan decides), with an error of at most (n_chan - 1) 2^-24
+ * sum_c |in| either way.
  * --------------------------------------------------------------------- */
 typedef struct fdas_dedisp_plan fdas_dedisp_plan;
 
@@ -526,7 +529,9 @@ typedef struct {
     double f_top_mhz, df_mhz, tsamp, dm_lo, dm_step;
     int32_t max_delay;        /* largest Delta(c, d)                           */
     int32_t tile_span;        /* largest delay spread over 32 consecutive DMs  */
-    int64_t workspace_bytes;  /* device memory the plan holds (delay table)   */
+    int64_t workspace_bytes;  /* device memory the plan holds (delay table and,
+                                 where channels are summed in groups, their
+                                 tables: 368 bytes a group and 32 trials)     */
 } fdas_dedisp_info;
 
 /* n_chan in [1, 65536], n_dm in [1, 65536], 1 <= n_out <= n_t,

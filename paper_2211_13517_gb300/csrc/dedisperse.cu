@@ -15,7 +15,8 @@
 // in FP64 with every operation rounded separately (no contraction), so they
 // are exactly those of the same formula evaluated in IEEE FP64 elsewhere.
 //
-// Kernel: a CTA owns 32 DM trials x 512 output samples.  Per batch of
+// Plain kernel (by channel groups: further down): a CTA owns 32 DM trials x 512
+// output samples.  Per batch of
 // channels it stages, for each channel, the window of input samples its 32
 // DMs read (512 + the spread of their delays) in shared memory by
 // asynchronous 4-byte copies (cp.async, zero-filled past n_t), double
