@@ -179,8 +179,8 @@ constexpr float kIbFactor = 0.61685027506808491f;   // (pi/4)^2
 // stage, two stages, and the plane is stored in FP32.
 //
 // kPool: also write the plane's maxima over boxes of 2 columns x one row block
-// (blocks of 3 to 5 rows of a chunk half, chunks[].ends), which the harmonic sum
-// by bounds reads: the cells are at hand here, and a separate pass over the
+// (blocks of at most 4 rows of a chunk half, chunks[].ends), which the harmonic
+// sum by bounds reads: the cells are at hand here, and a separate pass over the
 // plane takes 247 us at 2^22 bins x 193 rows BF16 (see pool_kernel).
 template <class P, int kMode, bool kPool>
 __global__ void __launch_bounds__(kTcThreads, 1)

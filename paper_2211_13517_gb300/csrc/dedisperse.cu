@@ -16,10 +16,9 @@
 // are exactly those of the same formula evaluated in IEEE FP64 elsewhere.
 //
 // Plain kernel (by channel groups: further down): a CTA owns 32 DM trials x 512
-// output samples.  Per batch of
-// channels it stages, for each channel, the window of input samples its 32
-// DMs read (512 + the spread of their delays) in shared memory by
-// asynchronous 4-byte copies (cp.async, zero-filled past n_t), double
+// output samples.  Per batch of channels it stages, for each channel, the window
+// of input samples its 32 DMs read (512 + the spread of their delays) in shared
+// memory by asynchronous 4-byte copies (cp.async, zero-filled past n_t), double
 // buffered so that the copies of the next batch run during the sums of this
 // one.  Warp w accumulates DMs 4w..4w+3, lane l the samples l + 32k (k < 16),
 // reading shared memory with consecutive lanes on consecutive words; where

@@ -3,15 +3,15 @@
 //
 // A 6-sigma crossing is rare (about one cell in 10^9 of noise), so almost
 // every sum only has to be shown not to cross.  The plane is reduced to its
-// maxima over boxes of 2 bins x one row block (3 to 5 template rows),
-// A[block][r/2], and a box of the top plane is compared through the maxima of
+// maxima over boxes of 2 bins x one row block (at most kPoolMaxRows = 4 template
+// rows), A[block][r/2], and a box of the top plane is compared through the maxima of
 // the boxes its harmonics read:
 //
 //   for every cell of the box and every stage,  S_h <= sum_j max(boxes of j).
 //
 // A box whose bound stays below every stage threshold holds no crossing.  The
 // cells of the others (about 7 in 10^4 boxes of noise at 6 sigma, 16
-// harmonics) are summed exactly, in the same stage order and FP32 rounding as
+// harmonics, z_step 1; more at coarser steps, see bounds_pay in plan.cu) are summed exactly, in the same stage order and FP32 rounding as
 // harmonic_dedup_kernel, and compared exactly, so the records are identical.
 // Neighbouring templates are strongly correlated, neighbouring bins are not:
 // pooling 2 bins x 4 rows passes 7e-4 of noise boxes, 4 bins x 2 rows 1.3e-2
@@ -564,7 +564,8 @@ fdas_status launch_bound_P(Plan &p, const void *plane, int buf, bool pooled, con
 
 }  // namespace
 
-// first rows of the row blocks (and n_z at the end): runs of about 4 rows
+// first rows of the row blocks (and n_z at the end): runs of 3 or 4 rows (of 1 or 2
+// for the smallest n_z)
 std::vector<int32_t> pool_blocks(int n_z) {
     std::vector<int32_t> out;
     const int nb = (n_z + 3) / 4;
