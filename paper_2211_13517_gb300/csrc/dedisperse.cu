@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kDdThreads, 2)
 // 6.63 ms below), its sums lie packed in shared memory (a place for the most
 // patterns of any group left room for 2 groups only: 7.04), and what a piece
 // reads again for each pattern stays in registers (7.35 without).
-// Measured: 1024 channels of 8-bit samples, 128 trials, 2^20 outputs 6.07 ms
+// Measured: 1024 channels of 8-bit samples, 128 trials, 2^20 outputs 5.90 ms
 // (plain kernel 18.7); 300 FP32 channels, 75 trials, 262181 outputs 0.60 ms
 // (1.32).
 // ---------------------------------------------------------------------------
