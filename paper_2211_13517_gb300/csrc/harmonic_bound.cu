@@ -10,9 +10,10 @@
 //   for every cell of the box and every stage,  S_h <= sum_j max(boxes of j).
 //
 // A box whose bound stays below every stage threshold holds no crossing.  The
-// cells of the others (about 7 in 10^4 boxes of noise at 6 sigma, 16
-// harmonics, z_step 1; more at coarser steps, see bounds_pay in plan.cu) are summed exactly, in the same stage order and FP32 rounding as
-// harmonic_dedup_kernel, and compared exactly, so the records are identical.
+// cells of the others (about 7 in 10^4 boxes of noise at 6 sigma, 16 harmonics,
+// z_step 1; more at coarser steps, see bounds_pay in plan.cu) are summed
+// exactly, in the same stage order and FP32 rounding as harmonic_dedup_kernel, and
+// compared exactly, so the records are identical.
 // Neighbouring templates are strongly correlated, neighbouring bins are not:
 // pooling 2 bins x 4 rows passes 7e-4 of noise boxes, 4 bins x 2 rows 1.3e-2
 // (measured on a noise plane, 193 templates, 16 harmonics, 6 sigma).
